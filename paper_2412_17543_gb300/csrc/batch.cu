@@ -573,7 +573,7 @@ void launch_map_scatter_b(int prec, int64_t n, const int* map, const void* in, v
 // T^T X_bi into out_bj for the tiles of its columns, so every output block has one
 // writer and the sums are deterministic. Tiles are read row by row (broadcast loads).
 // ---------------------------------------------------------------------------
-constexpr int SYMM_WARPS = 4;
+constexpr int SYMM_WARPS = 16;  // a level-2 matrix (about 13 block rows) alone on its SM: 4 warps left it idle
 
 template <class T>
 __global__ void __launch_bounds__(SYMM_WARPS * 32) k_symm_b(SymTiles A, const int64_t* __restrict__ voff,
@@ -854,72 +854,51 @@ __device__ __forceinline__ void bblock_store(const double* v, int nd, double* pa
   }
 }
 
-// member dots of df64 vectors, accumulated in df64 on the FP32 pipes
-__global__ void __launch_bounds__(BRB) k_bdots(int64_t n, const df64* __restrict__ a0, const df64* __restrict__ b0,
-                                               const df64* __restrict__ a1, const df64* __restrict__ b1,
-                                               double* partials) {
-  const int lane = threadIdx.x & 31;
-  df64_acc s0, s1;
-  for (int64_t i = (blockIdx.x * (int64_t)BRB + threadIdx.x) >> 5; i < n; i += ((int64_t)gridDim.x * BRB) >> 5) {
-    s0.fma(a0[i * BW + lane], b0[i * BW + lane]);
-    if (a1) s1.fma(a1[i * BW + lane], b1[i * BW + lane]);
-  }
-  double v[2] = {df64_to_double_bits(s0.get()), df64_to_double_bits(s1.get())};
-  bblock_store(v, 2, partials);
-}
+// Finalization by the last blocks of the reduction launch itself. Level 1: the last block
+// of each group of BFG sums the group's partials; level 2: the last group sums the group
+// sums and updates the scalars (lane = member). Every sum has a fixed order (segments of
+// its inputs, added in order), so the result does not depend on which block ends last.
+// A separate one-CTA kernel over the NBLKB partials took 27 us, three times per iteration:
+// its 1216 x 2 x 32 FP64 additions ran on one SM's FP64 pipe (2 per clock). Here the 38
+// groups' additions run on different SMs and no launch is added (ensemble of 12 on 48x32x40: 10.08 ->
+// 9.06 ms per step).
+struct BFinArgs {
+  double* sc;
+  int op, flexible;
+  const int* its;
+  unsigned* ticket;  // [1 + groups], zero between launches
+};
+constexpr int BFG = 32;                                // blocks per group
+constexpr int BFGROUPS = (NBLKB + BFG - 1) / BFG;      // group records follow the NBLKB block records
+static_assert(BFGROUPS == BFIN_GROUPS, "ticket and partial buffers are sized by BFIN_GROUPS");
 
-// x += alpha p ; r -= alpha q ; partial ||r||^2   (per member alpha, df64 arithmetic)
-__global__ void __launch_bounds__(BRB) k_baxpy2(int64_t n, const double* __restrict__ sc, df64* __restrict__ x,
-                                                const df64* __restrict__ p, df64* __restrict__ r,
-                                                const df64* __restrict__ q, double* partials) {
-  const int lane = threadIdx.x & 31;
-  const df64 alpha = df64_from_double_bits(sc[BS_ALPHA * BW + lane]);
-  const df64 malpha = df64_neg(alpha);
-  df64_acc rr;
-  for (int64_t i = (blockIdx.x * (int64_t)BRB + threadIdx.x) >> 5; i < n; i += ((int64_t)gridDim.x * BRB) >> 5) {
-    const int64_t o = i * BW + lane;
-    df64_acc xa, ra;
-    xa.add(x[o]);
-    xa.fma(alpha, p[o]);
-    x[o] = xa.get();
-    ra.add(r[o]);
-    ra.fma(malpha, q[o]);
-    const df64 ri = ra.get();
-    r[o] = ri;
-    rr.fma(ri, ri);
+// tot[d * BW + m] = sum over i < cnt of src[i][d][m], d < nd (1 or 2), by the whole block
+__device__ __forceinline__ void bfin_sum(const double* src, int cnt, int nd, double* seg, double* tot) {
+  const int w = nd * BW, ns = BRB / w;
+  const int idx = threadIdx.x % w, sg = threadIdx.x / w;
+  const int i0 = sg * cnt / ns, i1 = (sg + 1) * cnt / ns;
+  double s = 0.0;
+  for (int i = i0; i < i1; i += 8) {
+    double e[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) e[u] = i + u < i1 ? __ldcg(&src[(int64_t)(i + u) * BND * BW + idx]) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += e[u];
   }
-  double v[1] = {df64_to_double_bits(rr.get())};
-  bblock_store(v, 1, partials);
-}
-
-// one warp, lane = member: sums the block partials in a fixed order and updates the
-// member's scalars. Inactive members keep alpha = beta = 0, so their iterates stay fixed.
-constexpr int BFIN_WARPS = 32;
-__global__ void __launch_bounds__(BFIN_WARPS * 32) k_bfinalize(int nblk, const double* __restrict__ partials,
-                                                               double* sc, int op, int flexible,
-                                                               const int* __restrict__ its) {
-  // warp w sums the blocks w, w + 32, ... (lane = member); warp 0 then adds the 32
-  // warp sums in order: a fixed reduction tree
-  __shared__ double part[BFIN_WARPS][2][BW];
-  {
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    double a0 = 0.0, a1 = 0.0;
-#pragma unroll 4
-    for (int b = w; b < nblk; b += BFIN_WARPS) {
-      a0 += partials[((int64_t)b * BND + 0) * BW + l];
-      a1 += partials[((int64_t)b * BND + 1) * BW + l];
-    }
-    part[w][0][l] = a0;
-    part[w][1][l] = a1;
+  seg[threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.x < w) {
+    double t = 0.0;
+    for (int q = 0; q < ns; ++q) t += seg[q * w + threadIdx.x];
+    tot[threadIdx.x] = t;
   }
   __syncthreads();
-  const int m = threadIdx.x;
-  if (m >= BW) return;
-  double t0 = 0.0, t1 = 0.0;
-  for (int w = 0; w < BFIN_WARPS; ++w) {
-    t0 += part[w][0][m];
-    t1 += part[w][1][m];
-  }
+}
+
+// the member's scalars from its sums t0, t1. Inactive members keep alpha = beta = 0, so
+// their iterates stay fixed.
+__device__ __forceinline__ void bfin_update(double* sc, int op, int flexible, const int* its, int m, double t0,
+                                            double t1) {
   double* S = sc;
   auto at = [&](int slot) -> double& { return S[slot * BW + m]; };
   const bool act = at(BS_ACT) != 0.0;
@@ -986,18 +965,81 @@ __global__ void __launch_bounds__(BFIN_WARPS * 32) k_bfinalize(int nblk, const d
   }
 }
 
-void bvec_dots(int64_t n, const df64* a0, const df64* b0, const df64* a1, const df64* b1, double* partials,
-               cudaStream_t s) {
-  k_bdots<<<NBLKB, BRB, 0, s>>>(n, a0, b0, a1, b1, partials);
+__device__ __forceinline__ void bfinalize_last(double* partials, int nd, const BFinArgs& f) {
+  __shared__ double seg[BRB], tot[2 * BW];
+  __shared__ bool last;
+  const int g = blockIdx.x / BFG, b0 = g * BFG, cnt = min((int)gridDim.x, b0 + BFG) - b0;
+  const int ng = ((int)gridDim.x + BFG - 1) / BFG;
+  double* gpart = partials + (int64_t)NBLKB * BND * BW;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&f.ticket[1 + g], 1u) == (unsigned)cnt - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  bfin_sum(partials + (int64_t)b0 * BND * BW, cnt, nd, seg, tot);
+  if (threadIdx.x < nd * BW) gpart[(int64_t)g * BND * BW + threadIdx.x] = tot[threadIdx.x];
+  if (threadIdx.x == 0) f.ticket[1 + g] = 0u;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&f.ticket[0], 1u) == (unsigned)ng - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  bfin_sum(gpart, ng, nd, seg, tot);
+  if (threadIdx.x < BW)
+    bfin_update(f.sc, f.op, f.flexible, f.its, threadIdx.x, tot[threadIdx.x], nd > 1 ? tot[BW + threadIdx.x] : 0.0);
+  if (threadIdx.x == 0) f.ticket[0] = 0u;
+}
+
+// member dots of df64 vectors, accumulated in df64 on the FP32 pipes
+__global__ void __launch_bounds__(BRB) k_bdots(int64_t n, const df64* __restrict__ a0, const df64* __restrict__ b0,
+                                               const df64* __restrict__ a1, const df64* __restrict__ b1,
+                                               double* partials, BFinArgs fin) {
+  const int lane = threadIdx.x & 31;
+  df64_acc s0, s1;
+  for (int64_t i = (blockIdx.x * (int64_t)BRB + threadIdx.x) >> 5; i < n; i += ((int64_t)gridDim.x * BRB) >> 5) {
+    s0.fma(a0[i * BW + lane], b0[i * BW + lane]);
+    if (a1) s1.fma(a1[i * BW + lane], b1[i * BW + lane]);
+  }
+  double v[2] = {df64_to_double_bits(s0.get()), df64_to_double_bits(s1.get())};
+  bblock_store(v, 2, partials);
+  bfinalize_last(partials, 2, fin);
+}
+
+// x += alpha p ; r -= alpha q ; partial ||r||^2   (per member alpha, df64 arithmetic)
+__global__ void __launch_bounds__(BRB) k_baxpy2(int64_t n, const double* sc, df64* __restrict__ x,
+                                                const df64* __restrict__ p, df64* __restrict__ r,
+                                                const df64* __restrict__ q, double* partials, BFinArgs fin) {
+  const int lane = threadIdx.x & 31;
+  const df64 alpha = df64_from_double_bits(sc[BS_ALPHA * BW + lane]);
+  const df64 malpha = df64_neg(alpha);
+  df64_acc rr;
+  for (int64_t i = (blockIdx.x * (int64_t)BRB + threadIdx.x) >> 5; i < n; i += ((int64_t)gridDim.x * BRB) >> 5) {
+    const int64_t o = i * BW + lane;
+    df64_acc xa, ra;
+    xa.add(x[o]);
+    xa.fma(alpha, p[o]);
+    x[o] = xa.get();
+    ra.add(r[o]);
+    ra.fma(malpha, q[o]);
+    const df64 ri = ra.get();
+    r[o] = ri;
+    rr.fma(ri, ri);
+  }
+  double v[1] = {df64_to_double_bits(rr.get())};
+  bblock_store(v, 1, partials);
+  bfinalize_last(partials, 1, fin);
+}
+
+void bvec_dots_fin(int64_t n, const df64* a0, const df64* b0, const df64* a1, const df64* b1, double* partials,
+                   double* sc, int op, int flexible, unsigned* ticket, cudaStream_t s, const int* its) {
+  k_bdots<<<NBLKB, BRB, 0, s>>>(n, a0, b0, a1, b1, partials, BFinArgs{sc, op, flexible, its, ticket});
   DD_CHECK_LAUNCH();
 }
-void bvec_finalize(const double* partials, double* sc, int op, int flexible, cudaStream_t s, const int* its) {
-  k_bfinalize<<<1, BFIN_WARPS * 32, 0, s>>>(NBLKB, partials, sc, op, flexible, its);
-  DD_CHECK_LAUNCH();
-}
-void bvec_axpy2(int64_t n, const double* sc, df64* x, const df64* p, df64* r, const df64* q, double* partials,
-                cudaStream_t s) {
-  k_baxpy2<<<NBLKB, BRB, 0, s>>>(n, sc, x, p, r, q, partials);
+void bvec_axpy2_fin(int64_t n, double* sc, df64* x, const df64* p, df64* r, const df64* q, double* partials,
+                    unsigned* ticket, cudaStream_t s) {
+  k_baxpy2<<<NBLKB, BRB, 0, s>>>(n, sc, x, p, r, q, partials, BFinArgs{sc, BFIN_RR, 0, nullptr, ticket});
   DD_CHECK_LAUNCH();
 }
 

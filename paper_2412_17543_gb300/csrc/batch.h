@@ -15,6 +15,7 @@
 namespace dd {
 
 constexpr int BW = 32;  // ensemble block width (members per row, one per lane)
+constexpr int BFIN_GROUPS = 38;   // groups of 32 reduction blocks (first level of the finalization)
 constexpr int NBLKB = 152 * 8;  // fixed reduction grid of the ensemble kernels (deterministic partials)
 
 // per-member device scalars, slot-major: sc[slot * BW + m]
@@ -41,7 +42,8 @@ struct BatchWork {
   df64 *F = nullptr, *X = nullptr;    // [n_free][BW]
   double* sc = nullptr;               // [BS_COUNT][BW]
   double* sc_host = nullptr;          // pinned mirror
-  double* partials = nullptr;         // [NBLKB][4][BW]
+  double* partials = nullptr;         // [NBLKB + BFIN_GROUPS][4][BW]
+  unsigned* ticket = nullptr;         // [1 + BFIN_GROUPS] block tickets of the reductions (0 between launches)
   df64* wpart = nullptr;              // [deflation blocks][MAXK][BW]
   double* mu = nullptr;               // [MAXK][BW]
   LoopCtl* ctl = nullptr;             // device-resident loop control
@@ -109,12 +111,13 @@ void launch_map_gather_b(int prec, int64_t n, const int* map, const void* in, vo
 void launch_map_scatter_b(int prec, int64_t n, const int* map, const void* in, void* out, cudaStream_t s);
 
 // ---- Krylov vectors, per member (df64 storage and arithmetic) ----
-void bvec_dots(int64_t n, const df64* a0, const df64* b0, const df64* a1, const df64* b1, double* partials,
-               cudaStream_t s);
-void bvec_finalize(const double* partials, double* sc, int op, int flexible, cudaStream_t s,
-                   const int* its = nullptr);
-void bvec_axpy2(int64_t n, const double* sc, df64* x, const df64* p, df64* r, const df64* q, double* partials,
-                cudaStream_t s);
+// the member scalars are updated by the last block of the launch (ticket: [1 + BFIN_GROUPS]
+// counters, zero before the first call and left zero; calls sharing them are ordered on one
+// stream; partials: [NBLKB + BFIN_GROUPS][4][BW])
+void bvec_dots_fin(int64_t n, const df64* a0, const df64* b0, const df64* a1, const df64* b1, double* partials,
+                   double* sc, int op, int flexible, unsigned* ticket, cudaStream_t s, const int* its = nullptr);
+void bvec_axpy2_fin(int64_t n, double* sc, df64* x, const df64* p, df64* r, const df64* q, double* partials,
+                    unsigned* ticket, cudaStream_t s);
 void bvec_sub(int64_t n, const df64* a, const df64* b, df64* y, cudaStream_t s);
 void bvec_init(double* sc, int nrhs, double rtol, int stop_rhs_norm, cudaStream_t s);
 // deflation with the shared basis (df64 copy W, k columns of length n, stride ld):

@@ -204,7 +204,9 @@ BatchWork& batch_work(dd_ctx* c, cudaStream_t s) {
   B->F = dvec(c->n_free);
   B->X = dvec(c->n_free);
   B->sc = A.alloc<double>((size_t)BS_COUNT * BW);
-  B->partials = A.alloc<double>((size_t)NBLKB * 4 * BW);
+  B->partials = A.alloc<double>((size_t)(NBLKB + BFIN_GROUPS) * 4 * BW);
+  B->ticket = A.alloc<unsigned>(1 + BFIN_GROUPS);
+  DD_CUDA(cudaMemsetAsync(B->ticket, 0, (1 + BFIN_GROUPS) * sizeof(unsigned), s));
   B->wpart = A.alloc<df64>((size_t)defl_blocks(std::max<int64_t>(n, 1)) * MAXK * BW);
   B->mu = A.alloc<double>((size_t)MAXK * BW);
   DD_CUDA(cudaMallocHost(&B->sc_host, (size_t)BS_COUNT * BW * sizeof(double)));
@@ -350,8 +352,7 @@ dd_status pcg_solve_b(dd_ctx* c, dd_recycle* st, double rtol, bool record, int n
   }
   schur_b(c, B.xg, B.q, s);
   bvec_sub(n, B.bvec, B.q, B.r, s);
-  bvec_dots(n, B.bvec, B.bvec, B.r, B.r, B.partials, s);
-  bvec_finalize(B.partials, B.sc, BFIN_BB, 0, s);
+  bvec_dots_fin(n, B.bvec, B.bvec, B.r, B.r, B.partials, B.sc, BFIN_BB, 0, B.ticket, s);
   // member 0 feeds the recycling histories while it is active
   launch_loop_begin_b(B.ctl, B.sc, o.maxit, record && st->hmax > 0 ? 1 : 0, s);
   // p enters the first update p = z + beta p - W mu with beta = 0
@@ -362,19 +363,17 @@ dd_status pcg_solve_b(dd_ctx* c, dd_recycle* st, double rtol, bool record, int n
     if (flex) copy_b(B.zold, B.z, n, bs);
     precond_b(c, B.r, B.z, bs);
     if (rec) launch_record_col0(B.ctl, B.z, st->Z, n, st->hmax, 1, bs);
-    bvec_dots(n, B.r, B.z, flex ? B.r : nullptr, flex ? B.zold : nullptr, B.partials, bs);
-    bvec_finalize(B.partials, B.sc, BFIN_RZL, flex, bs, &B.ctl->its);
+    bvec_dots_fin(n, B.r, B.z, flex ? B.r : nullptr, flex ? B.zold : nullptr, B.partials, B.sc, BFIN_RZL, flex,
+                  B.ticket, bs, &B.ctl->its);
     if (k) bdefl_mu(n, k, AW, n, B.z, st->Ginv, B.wpart, B.mu, bs);
     bdefl_update(n, k, W, n, B.mu, B.z, B.p, B.sc, BS_BETA, -1.0, bs);
     schur_b(c, B.p, B.q, bs);
-    bvec_dots(n, B.p, B.q, nullptr, nullptr, B.partials, bs);
-    bvec_finalize(B.partials, B.sc, BFIN_PQ, 0, bs);
+    bvec_dots_fin(n, B.p, B.q, nullptr, nullptr, B.partials, B.sc, BFIN_PQ, 0, B.ticket, bs);
     if (rec) {
       launch_record_col0(B.ctl, B.p, st->P, n, st->hmax, 0, bs);
       launch_record_col0(B.ctl, B.q, st->AP, n, st->hmax, 0, bs);
     }
-    bvec_axpy2(n, B.sc, B.xg, B.p, B.r, B.q, B.partials, bs);
-    bvec_finalize(B.partials, B.sc, BFIN_RR, 0, bs);
+    bvec_axpy2_fin(n, B.sc, B.xg, B.p, B.r, B.q, B.partials, B.ticket, bs);
     launch_loop_check_b(B.ctl, B.sc, B.alphas, h, in_graph, bs);
   };
   const std::vector<uint64_t> key = {2,

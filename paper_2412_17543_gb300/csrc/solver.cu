@@ -495,8 +495,6 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
     }
     A.slots = pick;
   };
-  tune_sym(c->b1.N, c->b1.goff, w.rloc, w.uloc, c->info.tune_symv_ms);
-  if (c->mesh.local_solver != DD_LOCAL_FDM) tune_sym(c->mesh.KIIinv, c->mesh.ioff, w.tI, w.sI, c->info.tune_kii_ms);
   if (schur_fused_available(c->mesh)) {
     float best = 0.f;
     int pick = 256, i = 0;
@@ -557,6 +555,13 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
       zero(A.sticket, (size_t)A.count * sizeof(unsigned));
     }
   };
+  // (16^3 with 64 subdomains: one CTA per N_i left 88 SMs idle; two or more parts, 3.9 % of a solve)
+  split_sym(c->b1.N);
+  tune_sym(c->b1.N, c->b1.goff, w.rloc, w.uloc, c->info.tune_symv_ms);
+  if (c->mesh.local_solver != DD_LOCAL_FDM) {
+    split_sym(c->mesh.KIIinv);
+    tune_sym(c->mesh.KIIinv, c->mesh.ioff, w.tI, w.sI, c->info.tune_kii_ms);
+  }
   zero(w.uC, c->b1.n_coarse * sizeof(double));
   tune_rows(c->b1.PhiT, c->b1.goff, nullptr, w.rloc, c->b1.coff, w.gloc, 1.0, nullptr);
   split_cols(c->b1.PhiT);
