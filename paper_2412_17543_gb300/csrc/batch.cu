@@ -833,6 +833,96 @@ void launch_dense_mm(int prec, int n, const void* A, const void* x, void* y, cud
   DD_CHECK_LAUNCH();
 }
 
+// The explicit coarse operator times BW members. A block takes CM_ROWS rows, its eight warps
+// an eighth of the columns each (32 columns at a time: the rows' entries staged in shared
+// memory and read back as broadcast quads, the members' vectors coalesced from L2), and the
+// warps' sums are added in warp order.
+constexpr int CM_ROWS = 8;
+template <class T>
+struct alignas(16) Quad {
+  T v[4];
+};
+template <class T>
+__global__ void __launch_bounds__(256) k_coarse_mm(int n, const T* __restrict__ M, const T* __restrict__ x,
+                                                   T* __restrict__ y) {
+  __shared__ __align__(16) T as[8][CM_ROWS][32];
+  __shared__ T red[8][CM_ROWS][BW];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i0 = blockIdx.x * CM_ROWS;
+  const int chunks = (n + 31) / 32;
+  T acc[CM_ROWS];
+#pragma unroll
+  for (int r = 0; r < CM_ROWS; ++r) acc[r] = (T)0;
+  for (int ch = warp * chunks / 8; ch < (warp + 1) * chunks / 8; ++ch) {
+    const int j0 = ch * 32;
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < CM_ROWS; ++r)
+      as[warp][r][lane] = (i0 + r < n && j0 + lane < n) ? M[(int64_t)(i0 + r) * n + j0 + lane] : (T)0;
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 32; q += 4) {
+      T xv[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) xv[u] = j0 + q + u < n ? x[(int64_t)(j0 + q + u) * BW + lane] : (T)0;
+#pragma unroll
+      for (int r = 0; r < CM_ROWS; ++r) {
+        const Quad<T> a = *reinterpret_cast<const Quad<T>*>(&as[warp][r][q]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[r] = fma(a.v[u], xv[u], acc[r]);
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < CM_ROWS; ++r) red[warp][r][lane] = acc[r];
+  __syncthreads();
+  // 256 threads: row warp, member lane
+  if (i0 + warp < n) {
+    T s = red[0][warp][lane];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += red[w][warp][lane];
+    y[(int64_t)(i0 + warp) * BW + lane] = s;
+  }
+}
+void launch_coarse_mm(int prec, int n, const void* M, const void* x, void* y, cudaStream_t s) {
+  if (n == 0) return;
+  const int blocks = (n + CM_ROWS - 1) / CM_ROWS;
+  if (prec == DD_PREC_FP32)
+    k_coarse_mm<float><<<blocks, 256, 0, s>>>(n, (const float*)M, (const float*)x, (float*)y);
+  else
+    k_coarse_mm<double><<<blocks, 256, 0, s>>>(n, (const double*)M, (const double*)x, (double*)y);
+  DD_CHECK_LAUNCH();
+}
+
+template <class T>
+__global__ void k_unit_cols(int n, int j0, T* __restrict__ x) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t < (int64_t)n * BW) x[t] = t / BW == j0 + t % BW ? (T)1 : (T)0;
+}
+template <class T>
+__global__ void k_store_cols(int n, int j0, const T* __restrict__ u, T* __restrict__ M) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t i = t / BW;
+  const int j = j0 + (int)(t % BW);
+  if (i < n && j < n) M[i * n + j] = u[t];
+}
+void launch_unit_cols(int prec, int n, int j0, void* x, cudaStream_t s) {
+  const unsigned blocks = (unsigned)(((int64_t)n * BW + 255) / 256);
+  if (prec == DD_PREC_FP32)
+    k_unit_cols<float><<<blocks, 256, 0, s>>>(n, j0, (float*)x);
+  else
+    k_unit_cols<double><<<blocks, 256, 0, s>>>(n, j0, (double*)x);
+  DD_CHECK_LAUNCH();
+}
+void launch_store_cols(int prec, int n, int j0, const void* u, void* M, cudaStream_t s) {
+  const unsigned blocks = (unsigned)(((int64_t)n * BW + 255) / 256);
+  if (prec == DD_PREC_FP32)
+    k_store_cols<float><<<blocks, 256, 0, s>>>(n, j0, (const float*)u, (float*)M);
+  else
+    k_store_cols<double><<<blocks, 256, 0, s>>>(n, j0, (const double*)u, (double*)M);
+  DD_CHECK_LAUNCH();
+}
+
 // ---------------------------------------------------------------------------
 // Krylov vectors of the ensemble: per-member dots (lane = member, so a warp's rows
 // reduce without shuffles), fixed-order two-stage reductions, device-side stopping

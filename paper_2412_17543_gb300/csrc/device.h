@@ -161,6 +161,12 @@ struct DevLevel2 {
   int n3;
 };
 
+// Coarse spaces of at most this many dofs apply the level-2 BDDC as one explicit matrix
+// (built at setup). The recursive form is a chain of fourteen dependent launches of 2-8 us
+// each; the matrix costs its n^2 entries from L2 or HBM.
+constexpr int COARSE_DENSE_MAX = 4096;    // one vector: 67 MB of floats at most
+constexpr int COARSE_DENSE_MAX_B = 2048;  // ensembles: each block of 8 rows reads all members' vectors
+
 // Scratch buffers of the operators (device).
 struct Work {
   double* tI;      // [n_int] level-1 interior
@@ -213,6 +219,10 @@ void launch_coef_grad(const DevMesh& m, const double* x, const double* lam, doub
 void launch_coef_mismatch(const DevMesh& m, const double* coef, int log, double* part, int nblk, cudaStream_t s);
 void launch_scatter_recover(const DevMesh& m, const double* xg, const double* sI, double* x, cudaStream_t s);
 void launch_restrict(int64_t nflat, const int* gmap, const double* D, const double* r, double* rloc, cudaStream_t s);
+// the explicit coarse operator of small coarse spaces: y = M x, x_j = sum of the copies of the
+// local coarse vectors (x and the sums in the type of prec); xs: [n] scratch of that type
+void launch_coarse_gemv(int n, int prec, const void* M, const int* cptr, const int* cidx, const double* gloc,
+                        void* xs, double* y, cudaStream_t s);
 void launch_dense_gemv(int n, int prec, const void* A, const double* x, double* y, cudaStream_t s);
 // per item m: out[out_off[m]+i] = alpha * sum_j M_m[i][j] x_j (+ add[out_off[m]+i]),
 // x_j = in[in_map ? in_map[in_off[m]+j] : in_off[m]+j]

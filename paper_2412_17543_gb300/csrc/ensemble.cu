@@ -135,15 +135,41 @@ void select_shapes(dd_ctx* c, cudaStream_t s) {
   check_err(c, s);
 }
 
+// whether the ensemble applies the level-2 BDDC as the explicit matrix
+bool dense_coarse_b(const dd_ctx* c) { return c->KCd && c->b1.n_coarse <= COARSE_DENSE_MAX_B; }
+
 void select_ops(dd_ctx* c, cudaStream_t s) {
   BatchWork& B = *c->bw;
   select_shapes(c, s);
   select_op(c, BOP_N1, c->b1.N, c->b1.goff, B.rloc, B.uloc, c->b1.n_flat, s);
-  if (c->levels == 3) {
+  if (c->levels == 3 && !dense_coarse_b(c)) {
     const DevLevel2& L = c->l2;
     select_op(c, BOP_KII2, L.KIIinv, L.ioff, B.gI2, B.u0I2, L.n_int, s);
     select_op(c, BOP_N2, L.b.N, L.b.goff, B.rloc2, B.uloc2, L.b.n_flat, s);
   }
+}
+
+void* typed_vec(DeviceArena& A, int prec, int64_t rows) {
+  return prec == DD_PREC_FP32 ? (void*)A.alloc<float>((size_t)std::max<int64_t>(rows, 1) * BW)
+                              : (void*)A.alloc<double>((size_t)std::max<int64_t>(rows, 1) * BW);
+}
+
+// scratch of the level-2 BDDC
+void alloc_level2(dd_ctx* c, BatchWork& B) {
+  const DevLevel2& L = c->l2;
+  auto tvec = [&](int64_t rows) { return typed_vec(B.arena, L.b.prec, rows); };
+  B.gI2 = tvec(L.n_int);
+  B.u0I2 = tvec(L.n_int);
+  B.uI2 = tvec(L.n_int);
+  B.rl2 = tvec(L.b.n_flat);
+  B.rloc2 = tvec(L.b.n_flat);
+  B.uloc2 = tvec(L.b.n_flat);
+  B.vloc2 = tvec(L.b.n_flat);
+  B.r2 = tvec(L.b.n_gamma);
+  B.z2 = tvec(L.b.n_gamma);
+  B.gloc2 = tvec(L.b.n_cflat);
+  B.g3 = tvec(L.n3);
+  B.u3 = tvec(L.n3);
 }
 
 BatchWork& batch_work(dd_ctx* c, cudaStream_t s) {
@@ -152,7 +178,7 @@ BatchWork& batch_work(dd_ctx* c, cudaStream_t s) {
   // the packed panels once (kept by the context)
   ensure_tiles(c->arena, c->b1.N, s);
   if (c->mesh.local_solver != DD_LOCAL_FDM) ensure_tiles(c->arena, c->mesh.KIIinv, s);
-  if (c->levels == 3) {
+  if (c->levels == 3 && !dense_coarse_b(c)) {
     ensure_tiles(c->arena, c->l2.KIIinv, s);
     ensure_tiles(c->arena, c->l2.b.N, s);
   }
@@ -161,10 +187,7 @@ BatchWork& batch_work(dd_ctx* c, cudaStream_t s) {
   const DevMesh& m = c->mesh;
   const int64_t n = c->n_gamma;
   auto dvec = [&](int64_t rows) { return A.alloc<df64>((size_t)std::max<int64_t>(rows, 1) * BW); };
-  auto tvec = [&](int prec, int64_t rows) -> void* {
-    return prec == DD_PREC_FP32 ? (void*)A.alloc<float>((size_t)std::max<int64_t>(rows, 1) * BW)
-                                : (void*)A.alloc<double>((size_t)std::max<int64_t>(rows, 1) * BW);
-  };
+  auto tvec = [&](int prec, int64_t rows) { return typed_vec(A, prec, rows); };
   B->tI = dvec(m.n_int);
   B->sI = dvec(m.n_int);
   B->yloc = dvec(c->b1.n_flat);
@@ -178,22 +201,7 @@ BatchWork& batch_work(dd_ctx* c, cudaStream_t s) {
   B->gloc = tvec(pp, c->b1.n_cflat);
   B->gC = tvec(pp, c->b1.n_coarse);
   B->uC = tvec(pp, c->b1.n_coarse);
-  if (c->levels == 3) {
-    const DevLevel2& L = c->l2;
-    const int p2 = L.b.prec;
-    B->gI2 = tvec(p2, L.n_int);
-    B->u0I2 = tvec(p2, L.n_int);
-    B->uI2 = tvec(p2, L.n_int);
-    B->rl2 = tvec(p2, L.b.n_flat);
-    B->rloc2 = tvec(p2, L.b.n_flat);
-    B->uloc2 = tvec(p2, L.b.n_flat);
-    B->vloc2 = tvec(p2, L.b.n_flat);
-    B->r2 = tvec(p2, L.b.n_gamma);
-    B->z2 = tvec(p2, L.b.n_gamma);
-    B->gloc2 = tvec(p2, L.b.n_cflat);
-    B->g3 = tvec(p2, L.n3);
-    B->u3 = tvec(p2, L.n3);
-  }
+  if (c->levels == 3 && !dense_coarse_b(c)) alloc_level2(c, *B);
   B->xg = dvec(n);
   B->r = dvec(n);
   B->z = dvec(n);
@@ -318,11 +326,26 @@ void precond_b(dd_ctx* c, const df64* r, df64* z, cudaStream_t s) {
          [&](const void* g, void* u, cudaStream_t ss) {
            if (c->levels == 2)
              launch_dense_mm(c->b1.prec, c->b1.n_coarse, c->KCinv, g, u, ss);
+           else if (dense_coarse_b(c))
+             launch_coarse_mm(c->b1.prec, c->b1.n_coarse, c->KCd, g, u, ss);
            else
              level2_b(c, g, u, ss);
          },
          s);
 }
+
+// The scratch that the level-2 operators find through the context while the explicit matrix is
+// built; the context's own workspace and tile pointers are put back whatever happens.
+struct ScratchLevel2 {
+  dd_ctx* c;
+  BatchWork* bw;
+  DevLevel2 l2;
+  ScratchLevel2(dd_ctx* c_, BatchWork* tmp) : c(c_), bw(c_->bw), l2(c_->l2) { c->bw = tmp; }
+  ~ScratchLevel2() {
+    c->bw = bw;
+    c->l2 = l2;
+  }
+};
 
 void copy_b(df64* dst, const df64* src, int64_t rows, cudaStream_t s) {
   DD_CUDA(cudaMemcpyAsync(dst, src, (size_t)rows * BW * sizeof(df64), cudaMemcpyDeviceToDevice, s));
@@ -409,6 +432,36 @@ dd_status pcg_solve_b(dd_ctx* c, dd_recycle* st, double rtol, bool record, int n
 }
 
 }  // namespace
+
+// The level-2 BDDC of a small coarse space as one matrix: its columns from the operators
+// themselves, BW unit vectors at a time. On the 64^3 mesh (2863 coarse dofs) the coarse branch of one
+// preconditioner application was fourteen dependent launches; it is two now.
+void build_coarse_dense(dd_ctx* c, cudaStream_t s) {
+  const int n = c->b1.n_coarse, prec = c->b1.prec;
+  if (c->levels != 3 || n == 0 || n > COARSE_DENSE_MAX) return;
+  const size_t eb = prec == DD_PREC_FP32 ? 4 : 8;
+  const int npad = (std::max(c->l2.KIIinv.max_n, c->l2.b.N.max_n) + 31) / 32 * 32;
+  if ((size_t)npad * BW * eb > 227 * 1024) return;  // the CUDA-core tile kernel holds a matrix's vectors
+  BatchWork tmp;
+  alloc_level2(c, tmp);
+  void* x = typed_vec(tmp.arena, prec, n);
+  void* u = typed_vec(tmp.arena, prec, n);
+  void* M = eb == 4 ? (void*)c->arena.alloc<float>((size_t)n * n) : (void*)c->arena.alloc<double>((size_t)n * n);
+  {
+    ScratchLevel2 scope(c, &tmp);
+    ensure_tiles(tmp.arena, c->l2.KIIinv, s);
+    ensure_tiles(tmp.arena, c->l2.b.N, s);
+    for (int j0 = 0; j0 < n; j0 += BW) {
+      launch_unit_cols(prec, n, j0, x, s);
+      level2_b(c, x, u, s);
+      launch_store_cols(prec, n, j0, u, M, s);
+    }
+    DD_CUDA(cudaStreamSynchronize(s));
+  }
+  c->gCt = eb == 4 ? (void*)c->arena.alloc<float>(n) : (void*)c->arena.alloc<double>(n);
+  c->KCd = M;
+}
+
 }  // namespace dd
 
 using namespace dd;

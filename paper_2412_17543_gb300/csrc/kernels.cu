@@ -1267,6 +1267,72 @@ void launch_dense_gemv(int n, int prec, const void* A, const double* x, double* 
   DD_CHECK_LAUNCH();
 }
 
+// x_j = sum of the copies of coarse dof j, in the preconditioner's type
+template <class T>
+__global__ void k_coarse_gather(int n, const int* __restrict__ ptr, const int* __restrict__ idx,
+                                const double* __restrict__ loc, T* __restrict__ x) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  double s = 0.0;
+  for (int k = ptr[j]; k < ptr[j + 1]; ++k) s += loc[idx[k]];
+  x[j] = (T)s;
+}
+
+// y = M x for the explicit coarse operator (row-major n x n, warp per row, eight coalesced
+// loads in flight per lane, x in shared memory). Bound by the latency of one row and the n^2
+// entries: the products replace a chain of fourteen small launches on the critical path beside
+// the N_i product. Sums in the operator's type, as in the products they replace.
+constexpr int CG_WARPS = 8;
+template <class T>
+__global__ void __launch_bounds__(CG_WARPS * 32) k_coarse_gemv(int n, const T* __restrict__ M,
+                                                               const T* __restrict__ x, double* __restrict__ y) {
+  extern __shared__ __align__(16) unsigned char cg_smem[];
+  T* xs = reinterpret_cast<T*>(cg_smem);
+  for (int j = threadIdx.x; j < n; j += blockDim.x) xs[j] = x[j];
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = blockIdx.x * CG_WARPS + warp; i < n; i += gridDim.x * CG_WARPS) {
+    const T* a = M + (int64_t)i * n;
+    T acc[4] = {0, 0, 0, 0};
+    for (int j0 = 0; j0 < n; j0 += 32 * BG_CHUNK) {
+      T v[BG_CHUNK];
+#pragma unroll
+      for (int u = 0; u < BG_CHUNK; ++u) {
+        const int j = j0 + u * 32 + lane;
+        v[u] = j < n ? a[j] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < BG_CHUNK; ++u) {
+        const int j = j0 + u * 32 + lane;
+        if (j < n) acc[u & 3] = fma(v[u], xs[j], acc[u & 3]);
+      }
+    }
+    T sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) y[i] = (double)sum;
+  }
+}
+
+template <class T>
+static void coarse_gemv_go(int n, const T* M, const int* cptr, const int* cidx, const double* gloc, T* xs, double* y,
+                           cudaStream_t s) {
+  k_coarse_gather<T><<<(n + 127) / 128, 128, 0, s>>>(n, cptr, cidx, gloc, xs);
+  DD_CHECK_LAUNCH();
+  const int blocks = std::min(152 * 4, (n + CG_WARPS - 1) / CG_WARPS);
+  k_coarse_gemv<T><<<blocks, CG_WARPS * 32, (size_t)n * sizeof(T), s>>>(n, M, xs, y);
+  DD_CHECK_LAUNCH();
+}
+
+void launch_coarse_gemv(int n, int prec, const void* M, const int* cptr, const int* cidx, const double* gloc,
+                        void* xs, double* y, cudaStream_t s) {
+  if (n == 0) return;
+  if (prec == DD_PREC_FP32)
+    coarse_gemv_go<float>(n, (const float*)M, cptr, cidx, gloc, (float*)xs, y, s);
+  else
+    coarse_gemv_go<double>(n, (const double*)M, cptr, cidx, gloc, (double*)xs, y, s);
+}
+
 __global__ void k_map_gather(int64_t n, const int* __restrict__ map, const double* __restrict__ in,
                              double* __restrict__ out) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)

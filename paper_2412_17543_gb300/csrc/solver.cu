@@ -259,7 +259,8 @@ struct Fork {
   }
 };
 
-// BDDC of one level on an interface residual r -> z, with a coarse solver callback.
+// BDDC of one level on an interface residual r -> z, with a coarse solver callback (the local
+// coarse vectors gloc -> u_C, gC scratch).
 // The coarse correction (Phi_i^T D_i R_i r, the coarse solve, Phi_i u_C) does not depend on
 // the local products N_i D_i R_i r: with a fork it is issued on a high-priority side
 // stream, so that its short, latency-bound launches run while the N_i product streams from
@@ -271,8 +272,7 @@ void bddc_apply(dd_ctx* c, const DevBDDC& b, const double* r, double* z, double*
   launch_restrict(b.n_flat, b.gmap, b.D, r, rloc, s);
   cudaStream_t sc = fk.begin(s);
   launch_bgemv(b.PhiT, b.goff, nullptr, rloc, b.coff, gloc, 1.0, nullptr, sc);  // Phi_i^T D_i R_i r
-  launch_gather(b.n_coarse, b.cptr, b.cidx, gloc, nullptr, nullptr, gC, sc);
-  coarse(gC, uC, sc);
+  coarse(gloc, gC, uC, sc);
   launch_bgemv_t(b.PhiT, b.coff, b.cmap, uC, b.goff, vloc, 1.0, nullptr, sc);  // Phi_i R_Ci u_C
   {
     ProfScope pk(c, &b == &c->b1 ? DD_PROF_SYMV_N : DD_PROF_COUNT, s);
@@ -299,7 +299,10 @@ void level2_apply(dd_ctx* c, const double* g, double* u, cudaStream_t s) {
   launch_bgemv_t(L.E, L.ioff, nullptr, w.gI2, L.b.goff, w.rl2, -1.0, nullptr, s);  // -K_GI K_II^{-1} g_I
   launch_gather(L.b.n_gamma, L.b.gptr, L.b.gidx, w.rl2, g, L.gam_c64, w.r2, s);  // g[gam_c] + sum of copies
   bddc_apply(c, L.b, w.r2, w.z2, w.rloc2, w.uloc2, w.vloc2, w.gloc2, w.g3, w.u3,
-             [&](const double* g3, double* u3, cudaStream_t ss) { launch_dense_gemv(L.n3, L.b.prec, L.KC3inv, g3, u3, ss); },
+             [&](const double* gloc, double* g3, double* u3, cudaStream_t ss) {
+               launch_gather(L.b.n_coarse, L.b.cptr, L.b.cidx, gloc, nullptr, nullptr, g3, ss);
+               launch_dense_gemv(L.n3, L.b.prec, L.KC3inv, g3, u3, ss);
+             },
              s, f1);
   f0.end(s);
   launch_bgemv(L.E, L.b.goff, L.b.gmap, w.z2, L.ioff, w.uI2, -1.0, w.u0I2, s);  // u0 - K_II^{-1} K_IG z
@@ -311,9 +314,15 @@ void precond_apply(dd_ctx* c, const double* r, double* z, cudaStream_t s) {
   ProfScope ps(c, DD_PROF_PRECOND, s);
   Work& w = c->w;
   bddc_apply(c, c->b1, r, z, w.rloc, w.uloc, w.vloc, w.gloc, w.gC, w.uC,
-             [&](const double* g, double* u, cudaStream_t ss) {
+             [&](const double* gloc, double* g, double* u, cudaStream_t ss) {
+               const DevBDDC& b = c->b1;
+               if (c->KCd) {
+                 launch_coarse_gemv(b.n_coarse, b.prec, c->KCd, b.cptr, b.cidx, gloc, c->gCt, u, ss);
+                 return;
+               }
+               launch_gather(b.n_coarse, b.cptr, b.cidx, gloc, nullptr, nullptr, g, ss);
                if (c->levels == 2)
-                 launch_dense_gemv(c->b1.n_coarse, c->b1.prec, c->KCinv, g, u, ss);
+                 launch_dense_gemv(b.n_coarse, b.prec, c->KCinv, g, u, ss);
                else
                  level2_apply(c, g, u, ss);
              },
@@ -565,7 +574,7 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
   zero(w.uC, c->b1.n_coarse * sizeof(double));
   tune_rows(c->b1.PhiT, c->b1.goff, nullptr, w.rloc, c->b1.coff, w.gloc, 1.0, nullptr);
   split_cols(c->b1.PhiT);
-  if (c->levels == 3) {
+  if (c->levels == 3 && !c->KCd) {
     DevLevel2& L = c->l2;
     zero(w.z2, L.b.n_gamma * sizeof(double));
     zero(w.u0I2, L.n_int * sizeof(double));
@@ -870,6 +879,7 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
       for (auto& e : c->ev_aux) DD_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     }
     DD_CUDA(cudaStreamSynchronize(s));
+    build_coarse_dense(c.get(), s);
     {
       // algorithmic bytes of one K_II^{-1} application: the operator data read once and the
       // vectors in and out (dense: packed triangles; FDM: 1D eigenbases and D^{-1})
@@ -926,7 +936,9 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
         return b + 8.0 * (3.0 * (double)L.n_gamma + 6.0 * lf + 3.0 * lc);
       };
       double pb = level_bytes(H->l1, pp);
-      if (c->levels == 3) {
+      if (c->levels == 3 && c->KCd) {
+        pb += (double)H->l1.n_coarse * H->l1.n_coarse * (pp == DD_PREC_FP32 ? 4.0 : 8.0);
+      } else if (c->levels == 3) {
         const double eb = pp == DD_PREC_FP32 ? 4.0 : 8.0;
         pb += level_bytes(H->l2, pp);
         for (int j = 0; j < H->l2.S; ++j) {
