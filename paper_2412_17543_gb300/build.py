@@ -37,7 +37,7 @@ def _flags(src: str) -> list:
 
 def build(verbose: bool = False, force: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    headers = [os.path.join(SRC, f) for f in os.listdir(SRC) if f.endswith(".h")]
+    headers = [os.path.join(SRC, f) for f in os.listdir(SRC) if f.endswith((".h", ".cuh"))]
     headers.append(os.path.join(HERE, "..", "include", "dd_solver.h"))
     newest_header = max(os.path.getmtime(h) for h in headers)
     exe = nvcc()

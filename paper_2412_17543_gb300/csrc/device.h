@@ -218,16 +218,17 @@ void launch_coef_grad(const DevMesh& m, const double* x, const double* lam, doub
 // part[b] (b < nblk) = block maxima of |k_e - c_e| / |k_e| (c_e = exp(coef_e) when log)
 void launch_coef_mismatch(const DevMesh& m, const double* coef, int log, double* part, int nblk, cudaStream_t s);
 void launch_scatter_recover(const DevMesh& m, const double* xg, const double* sI, double* x, cudaStream_t s);
-void launch_restrict(int64_t nflat, const int* gmap, const double* D, const double* r, double* rloc, cudaStream_t s);
 // the explicit coarse operator of small coarse spaces: y = M x, x_j = sum of the copies of the
 // local coarse vectors (x and the sums in the type of prec); xs: [n] scratch of that type
 void launch_coarse_gemv(int n, int prec, const void* M, const int* cptr, const int* cidx, const double* gloc,
                         void* xs, double* y, cudaStream_t s);
+void launch_restrict(int64_t nflat, const int* gmap, const double* D, const double* r, double* rloc, cudaStream_t s);
 void launch_dense_gemv(int n, int prec, const void* A, const double* x, double* y, cudaStream_t s);
 // per item m: out[out_off[m]+i] = alpha * sum_j M_m[i][j] x_j (+ add[out_off[m]+i]),
-// x_j = in[in_map ? in_map[in_off[m]+j] : in_off[m]+j]
+// x_j = in[in_map ? in_map[in_off[m]+j] : in_off[m]+j], times in_scale[in_off[m]+j] if given
 void launch_bgemv(const BatchedRows& B, const int64_t* in_off, const int* in_map, const double* in,
-                  const int64_t* out_off, double* out, double alpha, const double* add, cudaStream_t s);
+                  const int64_t* out_off, double* out, double alpha, const double* add, cudaStream_t s,
+                  const double* in_scale = nullptr);
 // per item m: out[out_off[m]+j] = alpha * sum_i M_m[i][j] x_i (+ add[out_off[m]+j]) (transposed product)
 void launch_bgemv_t(const BatchedRows& B, const int64_t* in_off, const int* in_map, const double* in,
                     const int64_t* out_off, double* out, double alpha, const double* add, cudaStream_t s);

@@ -401,8 +401,6 @@ __global__ void __launch_bounds__(SYMV_WARPS * 32, 5) k_symv(SymTiles A, const i
   V* part = tv + maxpad;                                                      // [W][maxpad]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t vo = voff[m];
-  for (int i = threadIdx.x; i < npad; i += blockDim.x) tv[i] = (i < n) ? P::from_d(in[vo + i]) : P::from_d(0.0);
-  for (int i = threadIdx.x; i < SYMV_WARPS * npad; i += blockDim.x) part[(i / npad) * maxpad + (i % npad)] = P::from_d(0.0);
   if (lane == 0)
     for (int k = 0; k < SYMV_SLOTS; ++k) mbar_init(&bars[warp * SYMV_SLOTS + k], 1);
   fence_mbar_init();
@@ -423,6 +421,10 @@ __global__ void __launch_bounds__(SYMV_WARPS * 32, 5) k_symv(SymTiles A, const i
   };
   if (lane == 0)
     for (int k = 0; k < SYMV_SLOTS && k < mine; ++k) issue(k, k);
+  // the input is staged while the first copies fly
+  for (int i = threadIdx.x; i < npad; i += blockDim.x) tv[i] = (i < n) ? P::from_d(in[vo + i]) : P::from_d(0.0);
+  for (int i = threadIdx.x; i < SYMV_WARPS * npad; i += blockDim.x) part[(i / npad) * maxpad + (i % npad)] = P::from_d(0.0);
+  __syncthreads();
   V* mypart = part + warp * maxpad;
   bool ok = true;
   int k = 0;
@@ -1065,7 +1067,8 @@ __global__ void __launch_bounds__(256) k_bgemv(const int64_t* __restrict__ row0,
                                                const int64_t* __restrict__ in_off, const int* __restrict__ in_map,
                                                const double* __restrict__ in, const int64_t* __restrict__ out_off,
                                                double* __restrict__ out, double alpha,
-                                               const double* __restrict__ add, int rows_per_block) {
+                                               const double* __restrict__ add, int rows_per_block,
+                                               const double* __restrict__ in_scale) {
   extern __shared__ __align__(16) unsigned char bg_smem[];
   T* xs = reinterpret_cast<T*>(bg_smem);
   const int m = blockIdx.x;
@@ -1073,7 +1076,10 @@ __global__ void __launch_bounds__(256) k_bgemv(const int64_t* __restrict__ row0,
   const int r0 = blockIdx.y * rows_per_block;
   if (r0 >= R) return;
   const int64_t io = in_off[m];
-  for (int j = threadIdx.x; j < C; j += blockDim.x) xs[j] = (T)in[in_map ? in_map[io + j] : io + j];
+  for (int j = threadIdx.x; j < C; j += blockDim.x) {
+    const double v = in[in_map ? in_map[io + j] : io + j];
+    xs[j] = (T)(in_scale ? in_scale[io + j] * v : v);
+  }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r1 = min(R, r0 + rows_per_block);
@@ -1103,22 +1109,24 @@ __global__ void __launch_bounds__(256) k_bgemv(const int64_t* __restrict__ row0,
 
 template <class T>
 static void bgemv_go(const BatchedRows& B, const int64_t* in_off, const int* in_map, const double* in,
-                     const int64_t* out_off, double* out, double alpha, const double* add, cudaStream_t s) {
+                     const int64_t* out_off, double* out, double alpha, const double* add, cudaStream_t s,
+                     const double* in_scale) {
   size_t smem = (size_t)std::max(B.max_cols, 1) * sizeof(T);
   if (smem > 48 * 1024) max_smem(k_bgemv<T>, smem);
   const int rpb = std::max(8, B.rows_per_block);
   dim3 grid(B.count, (B.max_rows + rpb - 1) / rpb);
   k_bgemv<T><<<grid, 256, smem, s>>>(B.row0, B.cols, B.moff, static_cast<const T*>(B.data), in_off, in_map, in,
-                                      out_off, out, alpha, add, rpb);
+                                      out_off, out, alpha, add, rpb, in_scale);
 }
 
 void launch_bgemv(const BatchedRows& B, const int64_t* in_off, const int* in_map, const double* in,
-                  const int64_t* out_off, double* out, double alpha, const double* add, cudaStream_t s) {
+                  const int64_t* out_off, double* out, double alpha, const double* add, cudaStream_t s,
+                  const double* in_scale) {
   if (B.nrows == 0) return;
   if (B.prec == DD_PREC_FP32)
-    bgemv_go<float>(B, in_off, in_map, in, out_off, out, alpha, add, s);
+    bgemv_go<float>(B, in_off, in_map, in, out_off, out, alpha, add, s, in_scale);
   else
-    bgemv_go<double>(B, in_off, in_map, in, out_off, out, alpha, add, s);
+    bgemv_go<double>(B, in_off, in_map, in, out_off, out, alpha, add, s, in_scale);
   DD_CHECK_LAUNCH();
 }
 
@@ -1278,11 +1286,12 @@ __global__ void k_coarse_gather(int n, const int* __restrict__ ptr, const int* _
   x[j] = (T)s;
 }
 
-// y = M x for the explicit coarse operator (row-major n x n, warp per row, eight coalesced
+// y = M x for the explicit coarse operator (row-major n x n, warp per row, sixteen coalesced
 // loads in flight per lane, x in shared memory). Bound by the latency of one row and the n^2
 // entries: the products replace a chain of fourteen small launches on the critical path beside
 // the N_i product. Sums in the operator's type, as in the products they replace.
 constexpr int CG_WARPS = 8;
+constexpr int CG_CHUNK = 16;
 template <class T>
 __global__ void __launch_bounds__(CG_WARPS * 32) k_coarse_gemv(int n, const T* __restrict__ M,
                                                                const T* __restrict__ x, double* __restrict__ y) {
@@ -1294,15 +1303,15 @@ __global__ void __launch_bounds__(CG_WARPS * 32) k_coarse_gemv(int n, const T* _
   for (int i = blockIdx.x * CG_WARPS + warp; i < n; i += gridDim.x * CG_WARPS) {
     const T* a = M + (int64_t)i * n;
     T acc[4] = {0, 0, 0, 0};
-    for (int j0 = 0; j0 < n; j0 += 32 * BG_CHUNK) {
-      T v[BG_CHUNK];
+    for (int j0 = 0; j0 < n; j0 += 32 * CG_CHUNK) {
+      T v[CG_CHUNK];
 #pragma unroll
-      for (int u = 0; u < BG_CHUNK; ++u) {
+      for (int u = 0; u < CG_CHUNK; ++u) {
         const int j = j0 + u * 32 + lane;
         v[u] = j < n ? a[j] : T(0);
       }
 #pragma unroll
-      for (int u = 0; u < BG_CHUNK; ++u) {
+      for (int u = 0; u < CG_CHUNK; ++u) {
         const int j = j0 + u * 32 + lane;
         if (j < n) acc[u & 3] = fma(v[u], xs[j], acc[u & 3]);
       }

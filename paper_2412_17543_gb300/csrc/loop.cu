@@ -6,6 +6,7 @@
 
 #include "batch.h"
 #include "loop.h"
+#include "loop.cuh"
 #include "vecops.h"
 
 namespace dd {
@@ -39,29 +40,7 @@ __global__ void k_loop_gate(const LoopCtl* ctl, cudaGraphConditionalHandle h) {
 
 __global__ void k_loop_check(LoopCtl* ctl, const double* __restrict__ sc, double* alphas,
                              cudaGraphConditionalHandle h, int in_graph) {
-  const int its = ctl->its + 1;
-  ctl->its = its;
-  if (its - 1 < ctl->maxit) alphas[its - 1] = sc[SC_ALPHA];
-  ctl->nalpha = its;
-  int go = 1;
-  if (sc[SC_FLAG] != 0.0) {
-    ctl->status = LOOP_BREAKDOWN;
-    go = 0;
-  } else {
-    const double rel = sqrt(sc[SC_RR]) / ctl->ref;
-    ctl->rel = rel;
-    if (!isfinite(rel)) {
-      ctl->status = LOOP_BREAKDOWN;
-      go = 0;
-    } else if (rel < ctl->rtol) {
-      go = 0;
-    } else if (its >= ctl->maxit) {
-      ctl->status = LOOP_NOT_CONVERGED;
-      go = 0;
-    }
-  }
-  ctl->go = go;
-  if (in_graph) cudaGraphSetConditional(h, (unsigned)go);
+  loop_check(ctl, sc, alphas, h, in_graph);
 }
 
 __global__ void k_loop_begin_b(LoopCtl* ctl, const double* __restrict__ scb, int maxit, int rec0) {
@@ -96,11 +75,9 @@ __global__ void k_loop_check_b(LoopCtl* ctl, const double* __restrict__ scb, dou
   if (in_graph) cudaGraphSetConditional(h, (unsigned)go);
 }
 
-__global__ void k_record(const LoopCtl* __restrict__ ctl, const double* __restrict__ src, double* __restrict__ dst,
-                         int64_t n, int limit, int inclusive) {
-  const int its = ctl->its;
-  if (inclusive ? its > limit : its >= limit) return;
-  double* d = dst + (int64_t)its * n;
+__global__ void k_record(RecDst rec, const double* __restrict__ src, int64_t n) {
+  double* d = record_slot(rec, n);
+  if (!d) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     d[i] = src[i];
 }
@@ -134,11 +111,10 @@ void launch_loop_check_b(LoopCtl* ctl, const double* scb, double* alphas, cudaGr
   k_loop_check_b<<<1, 1, 0, s>>>(ctl, scb, alphas, h, in_graph ? 1 : 0);
   DD_CHECK_LAUNCH();
 }
-void launch_record(const LoopCtl* ctl, const double* src, double* dst, int64_t n, int limit, int inclusive,
-                   cudaStream_t s) {
+void launch_record(const RecDst& rec, const double* src, int64_t n, cudaStream_t s) {
   if (n == 0) return;
   const int64_t blocks = std::min<int64_t>((n + 255) / 256, 4 * 152);
-  k_record<<<(unsigned)blocks, 256, 0, s>>>(ctl, src, dst, n, limit, inclusive);
+  k_record<<<(unsigned)blocks, 256, 0, s>>>(rec, src, n);
   DD_CHECK_LAUNCH();
 }
 void launch_record_col0(const LoopCtl* ctl, const df64* src, double* dst, int64_t n, int limit, int inclusive,

@@ -29,19 +29,26 @@ struct LoopCtl {
   int nalpha;     // alphas recorded (single sequence: its)
 };
 
+// Where a kernel of the iteration records the vector it forms: dst + its * n when its < limit
+// (inclusive: its <= limit), its read on the device. dst null: nothing is recorded.
+struct RecDst {
+  const LoopCtl* ctl = nullptr;
+  double* dst = nullptr;
+  int limit = 0, inclusive = 0;
+};
+
 // stopping test of the single sequence before the first iteration (sc: the PCG scalars
 // after the initial residual; alphas are written per iteration by the check)
 void launch_loop_begin(LoopCtl* ctl, const double* sc, double rtol, int maxit, int stop_rhs_norm, cudaStream_t s);
-// end of one iteration: its += 1, alpha recorded, stop on breakdown, convergence or maxit
+// end of one iteration: its += 1, alpha recorded, stop on breakdown, convergence or maxit (a
+// launch of its own only after a re-orthogonalization; else the update of x and r ends with it)
 void launch_loop_check(LoopCtl* ctl, const double* sc, double* alphas, cudaGraphConditionalHandle h, bool in_graph,
                        cudaStream_t s);
 // ensemble: the members' device flags decide; member 0's alphas are recorded while it is active
 void launch_loop_begin_b(LoopCtl* ctl, const double* scb, int maxit, int rec0, cudaStream_t s);
 void launch_loop_check_b(LoopCtl* ctl, const double* scb, double* alphas, cudaGraphConditionalHandle h,
                          bool in_graph, cudaStream_t s);
-// dst + its * n <- src when its < limit (inclusive: its <= limit), its read on the device
-void launch_record(const LoopCtl* ctl, const double* src, double* dst, int64_t n, int limit, int inclusive,
-                   cudaStream_t s);
+void launch_record(const RecDst& rec, const double* src, int64_t n, cudaStream_t s);
 // member 0 of an interleaved df64 ensemble vector into dst + its * n, when ctl->rec0 and
 // its < limit (inclusive: its <= limit)
 void launch_record_col0(const LoopCtl* ctl, const df64* src, double* dst, int64_t n, int limit, int inclusive,

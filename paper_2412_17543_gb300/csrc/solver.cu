@@ -213,11 +213,10 @@ const void* upload_dense(DeviceArena& A, const std::vector<double>& M, int prec)
 // ---------------------------------------------------------------------------
 // operators
 // ---------------------------------------------------------------------------
-void schur_apply(dd_ctx* c, const double* x, double* y, cudaStream_t s) {
-  ProfScope ps(c, DD_PROF_SCHUR, s);
+// the local results y_i = S_i R_i x of the Schur operator, in c->w.yloc
+void schur_local(dd_ctx* c, const double* x, cudaStream_t s) {
   if (schur_fused_available(c->mesh)) {
     launch_schur_fused(c->mesh, x, c->w.yloc, s);
-    launch_gather(c->n_gamma, c->mesh.gptr, c->mesh.gidx, c->w.yloc, nullptr, nullptr, y, s);
     return;
   }
   launch_elem_interior(c->mesh, ELEM_SCHUR, x, nullptr, c->w.tI, s);
@@ -226,6 +225,11 @@ void schur_apply(dd_ctx* c, const double* x, double* y, cudaStream_t s) {
     launch_kii_apply(c->mesh, c->w.tI, c->w.sI, c->w.err, s);
   }
   launch_elem_interface(c->mesh, ELEM_SCHUR, x, c->w.sI, c->w.yloc, s);
+}
+
+void schur_apply(dd_ctx* c, const double* x, double* y, cudaStream_t s) {
+  ProfScope ps(c, DD_PROF_SCHUR, s);
+  schur_local(c, x, s);
   launch_gather(c->n_gamma, c->mesh.gptr, c->mesh.gidx, c->w.yloc, nullptr, nullptr, y, s);
 }
 
@@ -265,13 +269,16 @@ struct Fork {
 // the local products N_i D_i R_i r: with a fork it is issued on a high-priority side
 // stream, so that its short, latency-bound launches run while the N_i product streams from
 // HBM, and the two branches meet before the weighted gather. Each kernel computes the same
-// values in either order.
+// values in either order. Leaves the local results u_i (uloc) and Phi_i u_C (vloc); the caller
+// gathers them. The coarse branch reads r through the restriction D_i R_i itself and does not wait for
+// the restricted vector of the local products (which read it from there: taking it through the
+// interface map in each of their blocks cost them 7 %).
 template <class CoarseFn>
-void bddc_apply(dd_ctx* c, const DevBDDC& b, const double* r, double* z, double* rloc, double* uloc, double* vloc,
-                double* gloc, double* gC, double* uC, CoarseFn coarse, cudaStream_t s, const Fork& fk) {
-  launch_restrict(b.n_flat, b.gmap, b.D, r, rloc, s);
+void bddc_local(dd_ctx* c, const DevBDDC& b, const double* r, double* rloc, double* uloc, double* vloc, double* gloc, double* gC,
+                double* uC, CoarseFn coarse, cudaStream_t s, const Fork& fk) {
   cudaStream_t sc = fk.begin(s);
-  launch_bgemv(b.PhiT, b.goff, nullptr, rloc, b.coff, gloc, 1.0, nullptr, sc);  // Phi_i^T D_i R_i r
+  launch_restrict(b.n_flat, b.gmap, b.D, r, rloc, s);
+  launch_bgemv(b.PhiT, b.goff, b.gmap, r, b.coff, gloc, 1.0, nullptr, sc, b.D);  // Phi_i^T D_i R_i r
   coarse(gloc, gC, uC, sc);
   launch_bgemv_t(b.PhiT, b.coff, b.cmap, uC, b.goff, vloc, 1.0, nullptr, sc);  // Phi_i R_Ci u_C
   {
@@ -279,7 +286,6 @@ void bddc_apply(dd_ctx* c, const DevBDDC& b, const double* r, double* z, double*
     launch_symv(b.N, b.goff, rloc, uloc, c->w.err, s);
   }
   fk.end(s);
-  launch_wgather(b.n_gamma, b.gptr, b.gidx, b.D, uloc, vloc, z, s);
 }
 
 // three-level: BDDC for the whole coarse system K_C u = g (interior correction, interface BDDC,
@@ -298,22 +304,23 @@ void level2_apply(dd_ctx* c, const double* g, double* u, cudaStream_t s) {
   launch_symv(L.KIIinv, L.ioff, w.gI2, w.u0I2, w.err, s0);
   launch_bgemv_t(L.E, L.ioff, nullptr, w.gI2, L.b.goff, w.rl2, -1.0, nullptr, s);  // -K_GI K_II^{-1} g_I
   launch_gather(L.b.n_gamma, L.b.gptr, L.b.gidx, w.rl2, g, L.gam_c64, w.r2, s);  // g[gam_c] + sum of copies
-  bddc_apply(c, L.b, w.r2, w.z2, w.rloc2, w.uloc2, w.vloc2, w.gloc2, w.g3, w.u3,
+  bddc_local(c, L.b, w.r2, w.rloc2, w.uloc2, w.vloc2, w.gloc2, w.g3, w.u3,
              [&](const double* gloc, double* g3, double* u3, cudaStream_t ss) {
                launch_gather(L.b.n_coarse, L.b.cptr, L.b.cidx, gloc, nullptr, nullptr, g3, ss);
                launch_dense_gemv(L.n3, L.b.prec, L.KC3inv, g3, u3, ss);
              },
              s, f1);
+  launch_wgather(L.b.n_gamma, L.b.gptr, L.b.gidx, L.b.D, w.uloc2, w.vloc2, w.z2, s);
   f0.end(s);
   launch_bgemv(L.E, L.b.goff, L.b.gmap, w.z2, L.ioff, w.uI2, -1.0, w.u0I2, s);  // u0 - K_II^{-1} K_IG z
   launch_map_scatter(L.n_int, L.imap, w.uI2, u, s);
   launch_map_scatter(L.b.n_gamma, L.gam_c, w.z2, u, s);
 }
 
-void precond_apply(dd_ctx* c, const double* r, double* z, cudaStream_t s) {
-  ProfScope ps(c, DD_PROF_PRECOND, s);
+// the local results of the preconditioner, in c->w.uloc and c->w.vloc
+void precond_local(dd_ctx* c, const double* r, cudaStream_t s) {
   Work& w = c->w;
-  bddc_apply(c, c->b1, r, z, w.rloc, w.uloc, w.vloc, w.gloc, w.gC, w.uC,
+  bddc_local(c, c->b1, r, w.rloc, w.uloc, w.vloc, w.gloc, w.gC, w.uC,
              [&](const double* gloc, double* g, double* u, cudaStream_t ss) {
                const DevBDDC& b = c->b1;
                if (c->KCd) {
@@ -327,6 +334,12 @@ void precond_apply(dd_ctx* c, const double* r, double* z, cudaStream_t s) {
                  level2_apply(c, g, u, ss);
              },
              s, Fork{c->s_coarse, c->ev_fork, c->ev_join});
+}
+
+void precond_apply(dd_ctx* c, const double* r, double* z, cudaStream_t s) {
+  ProfScope ps(c, DD_PROF_PRECOND, s);
+  precond_local(c, r, s);
+  launch_wgather(c->n_gamma, c->b1.gptr, c->b1.gidx, c->b1.D, c->w.uloc, c->w.vloc, z, s);
 }
 
 // z = M^{-1} r as the PCG sees it: without a Dirichlet face the constant interface vector
@@ -486,6 +499,7 @@ constexpr int SYMV_WARPS_HOST = 4;  // warps per CTA of k_symv
 
 void tune_shapes(dd_ctx* c, cudaStream_t s) {
   Work& w = c->w;
+  DD_CUDA(cudaMemsetAsync(c->r, 0, c->n_gamma * sizeof(double), s));
   DD_CUDA(cudaMemsetAsync(w.rloc, 0, c->b1.n_flat * sizeof(double), s));
   DD_CUDA(cudaMemsetAsync(w.tI, 0, c->mesh.n_int * sizeof(double), s));
   DD_CUDA(cudaMemsetAsync(c->p, 0, c->n_gamma * sizeof(double), s));
@@ -523,13 +537,13 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
   // of the symmetric products
   auto zero = [&](void* p, size_t bytes) { if (p && bytes) DD_CUDA(cudaMemsetAsync(p, 0, bytes, s)); };
   auto tune_rows = [&](BatchedRows& B, const int64_t* in_off, const int* in_map, const double* in,
-                       const int64_t* out_off, double* out, double alpha, const double* add) {
+                       const int64_t* out_off, double* out, double alpha, const double* add, const double* scale) {
     if (B.count == 0) return;
     float best = 0.f;
     int pick = 32;
     for (int rpb : {32, 16, 8}) {
       B.rows_per_block = rpb;
-      const float t = time_launches([&] { launch_bgemv(B, in_off, in_map, in, out_off, out, alpha, add, s); }, s);
+      const float t = time_launches([&] { launch_bgemv(B, in_off, in_map, in, out_off, out, alpha, add, s, scale); }, s);
       if (rpb == 32 || t < best) {
         best = t;
         pick = rpb;
@@ -572,16 +586,16 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
     tune_sym(c->mesh.KIIinv, c->mesh.ioff, w.tI, w.sI, c->info.tune_kii_ms);
   }
   zero(w.uC, c->b1.n_coarse * sizeof(double));
-  tune_rows(c->b1.PhiT, c->b1.goff, nullptr, w.rloc, c->b1.coff, w.gloc, 1.0, nullptr);
+  tune_rows(c->b1.PhiT, c->b1.goff, c->b1.gmap, c->r, c->b1.coff, w.gloc, 1.0, nullptr, c->b1.D);
   split_cols(c->b1.PhiT);
   if (c->levels == 3 && !c->KCd) {
     DevLevel2& L = c->l2;
     zero(w.z2, L.b.n_gamma * sizeof(double));
     zero(w.u0I2, L.n_int * sizeof(double));
-    zero(w.rloc2, L.b.n_flat * sizeof(double));
+    zero(w.r2, L.b.n_gamma * sizeof(double));
     split_cols(L.E);
-    tune_rows(L.E, L.b.goff, L.b.gmap, w.z2, L.ioff, w.uI2, -1.0, w.u0I2);
-    tune_rows(L.b.PhiT, L.b.goff, nullptr, w.rloc2, L.b.coff, w.gloc2, 1.0, nullptr);
+    tune_rows(L.E, L.b.goff, L.b.gmap, w.z2, L.ioff, w.uI2, -1.0, w.u0I2, nullptr);
+    tune_rows(L.b.PhiT, L.b.goff, L.b.gmap, w.r2, L.b.coff, w.gloc2, 1.0, nullptr, L.b.D);
     split_cols(L.b.PhiT);
     split_sym(L.KIIinv);
     split_sym(L.b.N);
@@ -854,7 +868,7 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
     c->sc = A.alloc<double>(SC_COUNT);
     c->ctl = A.alloc<LoopCtl>(1);
     c->alphas = A.alloc<double>((size_t)opt->maxit);
-    c->partials = A.alloc<double>(NBLK * MAXDOT);
+    c->partials = A.alloc<double>(std::max(NBLK, NBLK_GATHER) * MAXDOT);
     c->wpart = A.alloc<double>((size_t)std::max<int64_t>(NBLK, defl_df_part_rows(c->n_gamma)) * MAXK);
     c->mu = A.alloc<double>(MAXK);
     c->fticket = A.alloc<unsigned>(1);
@@ -1430,10 +1444,20 @@ dd_status pcg_solve(dd_ctx* c, dd_recycle* st, double rtol, bool record, dd_stat
   // one iteration of Algorithm 1 in the order z = M^{-1} r, beta, p = z + beta p - W mu,
   // q = A p, alpha, x += alpha p, r -= alpha q, stopping test (first pass: beta = 0)
   auto body = [&](cudaStream_t bs, cudaGraphConditionalHandle h, bool in_graph) {
-    if (flex) DD_CUDA(cudaMemcpyAsync(c->zold, c->z, n * sizeof(double), cudaMemcpyDeviceToDevice, bs));
-    precond_z(c, c->r, c->z, bs);
-    if (rec) launch_record(c->ctl, c->z, st->Z, n, st->hmax, 1, bs);
-    {
+    const RecDst recz{c->ctl, rec ? st->Z : nullptr, st ? st->hmax : 0, 1};
+    const RecDst recp{c->ctl, rec ? st->P : nullptr, st ? st->hmax : 0, 0};
+    auto update_p = [&] {
+      if (Wf)
+        defl_update_f(n, k, Wf, n, c->mu, c->z, c->p, c->sc, SC_BETA, -1.0, bs);
+      else
+        defl_update_df(n, k, Wd, n, c->mu, c->z, c->p, c->sc, SC_BETA, -1.0, bs);
+    };
+    const RecDst recq{c->ctl, rec ? st->AP : nullptr, st ? st->hmax : 0, 0};
+    if (c->neumann) {
+      // z is made mean-free before anything reads it
+      if (flex) DD_CUDA(cudaMemcpyAsync(c->zold, c->z, n * sizeof(double), cudaMemcpyDeviceToDevice, bs));
+      precond_z(c, c->r, c->z, bs);
+      if (rec) launch_record(recz, c->z, n, bs);
       // the deflation dots (AW)^T z and the Krylov dots r^T z (r^T z_old) only read z: the
       // former run on the side stream while the latter finalize beta on the main stream
       ProfScope pd(c, k ? DD_PROF_DEFL : DD_PROF_COUNT, bs);
@@ -1443,25 +1467,33 @@ dd_status pcg_solve(dd_ctx* c, dd_recycle* st, double rtol, bool record, dd_stat
       vec_dots_fin(n, c->r, c->z, flex ? c->r : nullptr, flex ? c->zold : nullptr, c->partials, c->sc, FIN_RZL, flex,
                    c->fticket, bs, &c->ctl->its);
       fk.end(bs);
-      if (Wf)
-        defl_update_f(n, k, Wf, n, c->mu, c->z, c->p, c->sc, SC_BETA, -1.0, bs);
-      else
-        defl_update_df(n, k, Wd, n, c->mu, c->z, c->p, c->sc, SC_BETA, -1.0, bs);
+      update_p();
+    } else {
+      {
+        ProfScope ps(c, DD_PROF_PRECOND, bs);
+        precond_local(c, c->r, bs);
+        vec_wgather_rz(n, c->b1.gptr, c->b1.gidx, c->b1.D, c->w.uloc, c->w.vloc, c->r, c->z, flex, c->partials, c->sc,
+                       &c->ctl->its, c->fticket, recz, bs);
+      }
+      ProfScope pd(c, k ? DD_PROF_DEFL : DD_PROF_COUNT, bs);
+      if (k) defl_mu_df(n, k, AWd, n, c->z, st->Ginv, c->wpart, c->mu, c->wticket, bs);
+      update_p();
     }
-    schur_apply(c, c->p, c->q, bs);
-    vec_dots_fin(n, c->p, c->q, nullptr, nullptr, c->partials, c->sc, FIN_PQ, 0, c->fticket, bs);
-    if (rec) {
-      launch_record(c->ctl, c->p, st->P, n, st->hmax, 0, bs);
-      launch_record(c->ctl, c->q, st->AP, n, st->hmax, 0, bs);
+    {
+      ProfScope ps(c, DD_PROF_SCHUR, bs);
+      schur_local(c, c->p, bs);
+      vec_gather_pq(n, c->mesh.gptr, c->mesh.gidx, c->w.yloc, c->p, c->q, c->partials, c->sc, c->fticket, recp, recq,
+                    bs);
     }
-    vec_axpy2_fin(n, c->sc, c->xg, c->p, c->r, c->q, c->partials, c->fticket, bs);
+    const IterEnd end{reo ? nullptr : c->ctl, c->alphas, h, in_graph ? 1 : 0};
+    vec_axpy2_fin(n, c->sc, c->xg, c->p, c->r, c->q, c->partials, c->fticket, end, bs);
     if (reo) {
       // r -= W (W^T W)^{-1} W^T r  (Algorithm 1, optional re-orthogonalization), then ||r||^2 again
       defl_mu_df(n, k, Wd, n, c->r, st->WWinv, c->wpart, c->mu, c->wticket, bs);
       defl_update_df(n, k, Wd, n, c->mu, nullptr, c->r, c->sc, -1, -1.0, bs);
       vec_dots_fin(n, c->r, c->r, nullptr, nullptr, c->partials, c->sc, FIN_RR, 0, c->fticket, bs);
+      launch_loop_check(c->ctl, c->sc, c->alphas, h, in_graph, bs);
     }
-    launch_loop_check(c->ctl, c->sc, c->alphas, h, in_graph, bs);
   };
   // everything the captured body bakes into its launches
   const std::vector<uint64_t> key = {1,

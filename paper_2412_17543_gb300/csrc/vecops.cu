@@ -5,6 +5,7 @@
 // (eq. 15).
 #include <algorithm>
 
+#include "loop.cuh"
 #include "vecops.h"
 
 namespace dd {
@@ -29,26 +30,12 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[ND], double* part
   }
 }
 
-// single-block finalization: sums the partials in a fixed order (a warp per dot product,
-// fixed lane assignment and shuffle tree) and updates the scalars. CG: the partials were
-// written by other blocks of the same launch (read through L2).
-template <bool CG>
-__device__ __forceinline__ void finalize_block(int nblk, const double* partials, double* sc, int op, int flexible,
-                                               const int* its) {
-  __shared__ double tot[3];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp < 3) {
-    double s = 0.0;
-    for (int b = lane; b < nblk; b += 32) s += CG ? __ldcg(&partials[b * MAXDOT + warp]) : partials[b * MAXDOT + warp];
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) tot[warp] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
+// the PCG scalars from the sums t0, t1 of one reduction (one thread)
+__device__ __forceinline__ void fin_update(double t0, double t1, double* sc, int op, int flexible, const int* its) {
   if (op == FIN_RZL) op = *its == 0 ? FIN_RZ0 : FIN_RZ;  // device-resident loop: first iteration or not
   switch (op) {
     case FIN_PQ: {
-      double pq = tot[0];
+      double pq = t0;
       sc[SC_PQ] = pq;
       if (!(pq > 0.0) || !isfinite(pq) || !isfinite(sc[SC_RZ])) {
         sc[SC_FLAG] = 1.0;
@@ -59,15 +46,15 @@ __device__ __forceinline__ void finalize_block(int nblk, const double* partials,
       break;
     }
     case FIN_RR:
-      sc[SC_RR] = tot[0];
-      if (!isfinite(tot[0])) sc[SC_FLAG] = 1.0;
+      sc[SC_RR] = t0;
+      if (!isfinite(t0)) sc[SC_FLAG] = 1.0;
       break;
     case FIN_RZ0:
-      sc[SC_RZ] = tot[0];
-      if (!(tot[0] > 0.0) || !isfinite(tot[0])) sc[SC_FLAG] = 1.0;
+      sc[SC_RZ] = t0;
+      if (!(t0 > 0.0) || !isfinite(t0)) sc[SC_FLAG] = 1.0;
       break;
     case FIN_RZ: {
-      double rz_new = tot[0], rz_old_z = tot[1];
+      double rz_new = t0, rz_old_z = t1;
       double num = flexible ? (rz_new - rz_old_z) : rz_new;
       double rz = sc[SC_RZ];
       sc[SC_BETA] = (rz != 0.0) ? num / rz : 0.0;
@@ -76,12 +63,31 @@ __device__ __forceinline__ void finalize_block(int nblk, const double* partials,
       break;
     }
     case FIN_BB:
-      sc[SC_BB] = tot[0];
-      sc[SC_RR] = tot[1];
+      sc[SC_BB] = t0;
+      sc[SC_RR] = t1;
       break;
     default:
       break;
   }
+}
+
+// single-block finalization: sums the partials in a fixed order (a warp per dot product,
+// fixed lane assignment and shuffle tree) and updates the scalars. CG: the partials were
+// written by other blocks of the same launch (read through L2).
+template <bool CG>
+__device__ __forceinline__ void finalize_block(int nblk, const double* partials, double* sc, int op, int flexible,
+                                               const int* its) {
+  __shared__ double tot[3];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp < 3) {
+    double s = 0.0;
+#pragma unroll 8
+    for (int b = lane; b < nblk; b += 32) s += CG ? __ldcg(&partials[b * MAXDOT + warp]) : partials[b * MAXDOT + warp];
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) tot[warp] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) fin_update(tot[0], tot[1], sc, op, flexible, its);
 }
 
 __global__ void k_finalize(int nblk, const double* __restrict__ partials, double* sc, int op, int flexible,
@@ -96,6 +102,7 @@ struct FinArgs {
   int op, flexible;
   const int* its;
   unsigned* ticket;
+  IterEnd end;
 };
 __device__ __forceinline__ void finalize_last(const double* partials, const FinArgs& f) {
   __shared__ bool last;
@@ -107,6 +114,7 @@ __device__ __forceinline__ void finalize_last(const double* partials, const FinA
   __threadfence();
   if (threadIdx.x == 0) *f.ticket = 0u;
   finalize_block<true>((int)gridDim.x, partials, f.sc, f.op, f.flexible, f.its);
+  if (f.end.ctl && threadIdx.x == 0) loop_check(f.end.ctl, f.sc, f.end.alphas, f.end.h, f.end.in_graph);
 }
 
 // partial dots: d0 = a0.b0, d1 = a1.b1, d2 = a2.b2 (null pairs skipped); FIN: the last
@@ -126,9 +134,8 @@ __global__ void __launch_bounds__(RB) k_dots(int64_t n, const double* __restrict
   if (FIN) finalize_last(partials, fin);
 }
 
-// x += alpha p ; r -= alpha q ; partial ||r||^2 (FIN: the last block finalizes)
-template <bool FIN>
-__global__ void __launch_bounds__(RB) k_axpy2(int64_t n, const double* __restrict__ sc, double* __restrict__ x,
+// x += alpha p ; r -= alpha q ; ||r||^2, finalized by the last block, which may end the iteration
+__global__ void __launch_bounds__(RB) k_axpy2(int64_t n, const double* sc, double* __restrict__ x,
                                               const double* __restrict__ p, double* __restrict__ r,
                                               const double* __restrict__ q, double* partials, FinArgs fin) {
   const double alpha = sc[SC_ALPHA];
@@ -140,7 +147,91 @@ __global__ void __launch_bounds__(RB) k_axpy2(int64_t n, const double* __restric
     v[0] = fma(ri, ri, v[0]);
   }
   block_reduce_store<1>(v, partials);
-  if (FIN) finalize_last(partials, fin);
+  finalize_last(partials, fin);
+}
+
+// z, its record and the Krylov dots that follow in one pass: z_old is read where z is written, so
+// flexible PCG needs no copy of it (128^3: 7 us), and z and r are not read again
+__global__ void __launch_bounds__(RB) k_wgather_rz(int64_t n, const int* __restrict__ ptr,
+                                                   const int* __restrict__ idx, const double* __restrict__ D,
+                                                   const double* __restrict__ uloc, const double* __restrict__ vloc,
+                                                   const double* __restrict__ r, double* __restrict__ z, int flexible,
+                                                   double* partials, RecDst recz, FinArgs fin) {
+  double v[2] = {0.0, 0.0};
+  double* rz = record_slot(recz, n);
+  for (int64_t g = blockIdx.x * (int64_t)RB + threadIdx.x; g < n; g += (int64_t)gridDim.x * RB) {
+    double acc = 0.0;
+    const int k1 = ptr[g + 1];
+    const double rv = r[g], zo = flexible ? z[g] : 0.0;
+    for (int k = ptr[g]; k < k1; k += 4) {
+      int j[4];
+      double d[4], e[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) j[u] = k + u < k1 ? idx[k + u] : -1;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        d[u] = j[u] >= 0 ? D[j[u]] : 0.0;
+        e[u] = j[u] >= 0 ? uloc[j[u]] + vloc[j[u]] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc = fma(d[u], e[u], acc);
+    }
+    z[g] = acc;
+    if (rz) rz[g] = acc;
+    v[0] = fma(rv, acc, v[0]);
+    v[1] = fma(rv, zo, v[1]);
+  }
+  block_reduce_store<2>(v, partials);
+  finalize_last(partials, fin);
+}
+void vec_wgather_rz(int64_t n, const int* ptr, const int* idx, const double* D, const double* uloc,
+                    const double* vloc, const double* r, double* z, int flexible, double* partials, double* sc,
+                    const int* its, unsigned* ticket, const RecDst& recz, cudaStream_t s) {
+  const int blocks = (int)std::min<int64_t>(NBLK_GATHER, std::max<int64_t>(1, (n + RB - 1) / RB));
+  k_wgather_rz<<<blocks, RB, 0, s>>>(n, ptr, idx, D, uloc, vloc, r, z, flexible, partials, recz,
+                                     FinArgs{sc, FIN_RZL, flexible, its, ticket, IterEnd{}});
+  DD_CHECK_LAUNCH();
+}
+
+// q = sum of the copies of loc, p^T q: the gather of the Schur operator, the record of p and q and the
+// dot product that follows in one pass (p and q are not read again; one launch instead of four)
+__global__ void __launch_bounds__(RB) k_gather_pq(int64_t n, const int* __restrict__ ptr, const int* __restrict__ idx,
+                                                  const double* __restrict__ loc, const double* __restrict__ p,
+                                                  double* __restrict__ q, double* partials, RecDst recp, RecDst recq,
+                                                  FinArgs fin) {
+  double v[1] = {0.0};
+  double* rp = record_slot(recp, n);
+  double* rq = record_slot(recq, n);
+  for (int64_t g = blockIdx.x * (int64_t)RB + threadIdx.x; g < n; g += (int64_t)gridDim.x * RB) {
+    double s = 0.0;
+    const int k1 = ptr[g + 1];
+    // four copies' indices, then their values: two dependent loads per four copies
+    for (int k = ptr[g]; k < k1; k += 4) {
+      int j[4];
+      double e[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) j[u] = k + u < k1 ? idx[k + u] : -1;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) e[u] = j[u] >= 0 ? loc[j[u]] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s += e[u];
+    }
+    const double pv = p[g];
+    q[g] = s;
+    if (rp) rp[g] = pv;
+    if (rq) rq[g] = s;
+    v[0] = fma(pv, s, v[0]);
+  }
+  block_reduce_store<1>(v, partials);
+  finalize_last(partials, fin);
+}
+void vec_gather_pq(int64_t n, const int* ptr, const int* idx, const double* loc, const double* p, double* q,
+                   double* partials, double* sc, unsigned* ticket, const RecDst& recp, const RecDst& recq,
+                   cudaStream_t s) {
+  const int blocks = (int)std::min<int64_t>(NBLK_GATHER, std::max<int64_t>(1, (n + RB - 1) / RB));
+  k_gather_pq<<<blocks, RB, 0, s>>>(n, ptr, idx, loc, p, q, partials, recp, recq,
+                                    FinArgs{sc, FIN_PQ, 0, nullptr, ticket, IterEnd{}});
+  DD_CHECK_LAUNCH();
 }
 
 void vec_dots(int64_t n, const double* a0, const double* b0, const double* a1, const double* b1, const double* a2,
@@ -152,21 +243,16 @@ void vec_dots_fin(int64_t n, const double* a0, const double* b0, const double* a
                   double* partials, double* sc, int op, int flexible, unsigned* ticket, cudaStream_t s,
                   const int* its) {
   k_dots<true><<<NBLK, RB, 0, s>>>(n, a0, b0, a1, b1, nullptr, nullptr, partials,
-                                   FinArgs{sc, op, flexible, its, ticket});
+                                   FinArgs{sc, op, flexible, its, ticket, IterEnd{}});
   DD_CHECK_LAUNCH();
 }
 void vec_finalize(const double* partials, double* sc, int op, int flexible, cudaStream_t s, const int* its) {
   k_finalize<<<1, 96, 0, s>>>(NBLK, partials, sc, op, flexible, its);
   DD_CHECK_LAUNCH();
 }
-void vec_axpy2(int64_t n, const double* sc, double* x, const double* p, double* r, const double* q, double* partials,
-               cudaStream_t s) {
-  k_axpy2<false><<<NBLK, RB, 0, s>>>(n, sc, x, p, r, q, partials, FinArgs{});
-  DD_CHECK_LAUNCH();
-}
 void vec_axpy2_fin(int64_t n, double* sc, double* x, const double* p, double* r, const double* q, double* partials,
-                   unsigned* ticket, cudaStream_t s) {
-  k_axpy2<true><<<NBLK, RB, 0, s>>>(n, sc, x, p, r, q, partials, FinArgs{sc, FIN_RR, 0, nullptr, ticket});
+                   unsigned* ticket, const IterEnd& end, cudaStream_t s) {
+  k_axpy2<<<NBLK, RB, 0, s>>>(n, sc, x, p, r, q, partials, FinArgs{sc, FIN_RR, 0, nullptr, ticket, end});
   DD_CHECK_LAUNCH();
 }
 
@@ -346,6 +432,7 @@ __global__ void __launch_bounds__(RB) k_wdots8(int64_t n, int64_t rows, int k, c
   __threadfence();
   wd_reduce(gpart, ng, k, part, d);
   const int t = threadIdx.x;
+  if (t == 0) ticket[0] = 0u;
   const int ns = max(1, min(8, RB / k));
   if (t < ns * k) {
     // row a of Ginv over the c-segment sg, all loads in flight
@@ -368,7 +455,6 @@ __global__ void __launch_bounds__(RB) k_wdots8(int64_t n, int64_t rows, int k, c
     for (int sg = 0; sg < ns; ++sg) sum += part[sg * k + t];
     mu[t] = sum;
   }
-  if (t == 0) ticket[0] = 0u;
 }
 
 void defl_mu_df(int64_t n, int k, const df64* V, int64_t ld, const double* v, const double* Ginv, double* wpart,

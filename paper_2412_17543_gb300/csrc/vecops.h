@@ -4,12 +4,14 @@
 #include <stdint.h>
 
 #include "common.h"
+#include "loop.h"
 
 namespace dd {
 
 constexpr int NBLK = 304;   // reduction grid: 2 blocks per SM of GB300 (fixed => deterministic sums)
 constexpr int MAXDOT = 4;   // dot products per partial record
 constexpr int MAXK = 128;   // maximum deflation basis size
+constexpr int NBLK_GATHER = 608;   // reduction grid of the gather that ends with a dot product (four blocks per SM)
 
 // device scalar slots of PCG
 enum {
@@ -22,15 +24,30 @@ void vec_dots(int64_t n, const double* a0, const double* b0, const double* a1, c
               const double* b2, double* partials, cudaStream_t s);
 void vec_finalize(const double* partials, double* sc, int op, int flexible, cudaStream_t s,
                   const int* its = nullptr);
-void vec_axpy2(int64_t n, const double* sc, double* x, const double* p, double* r, const double* q, double* partials,
-               cudaStream_t s);
 // the same with vec_finalize done by the last block of the launch (ticket: a device counter,
 // zero between launches; the calls sharing one ticket must be ordered on one stream)
 void vec_dots_fin(int64_t n, const double* a0, const double* b0, const double* a1, const double* b1,
                   double* partials, double* sc, int op, int flexible, unsigned* ticket, cudaStream_t s,
                   const int* its = nullptr);
+// x += alpha p, r -= alpha q, ||r||^2; with check the last block also ends the iteration
+// (loop_check), else the caller does
+struct IterEnd {
+  LoopCtl* ctl = nullptr;  // null: no check
+  double* alphas = nullptr;
+  cudaGraphConditionalHandle h{};
+  int in_graph = 0;
+};
 void vec_axpy2_fin(int64_t n, double* sc, double* x, const double* p, double* r, const double* q, double* partials,
-                   unsigned* ticket, cudaStream_t s);
+                   unsigned* ticket, const IterEnd& end, cudaStream_t s);
+// z = sum over copies of D (u + v) (eq. 7), recorded, with r^T z and (flexible) r^T z_old, z_old the z it
+// replaces, and beta (FIN_RZL) in one launch
+void vec_wgather_rz(int64_t n, const int* ptr, const int* idx, const double* D, const double* uloc,
+                    const double* vloc, const double* r, double* z, int flexible, double* partials, double* sc,
+                    const int* its, unsigned* ticket, const RecDst& recz, cudaStream_t s);
+// q = sum of the interface copies of loc, p^T q and alpha (FIN_PQ) in one launch; p and q recorded
+void vec_gather_pq(int64_t n, const int* ptr, const int* idx, const double* loc, const double* p, double* q,
+                   double* partials, double* sc, unsigned* ticket, const RecDst& recp, const RecDst& recq,
+                   cudaStream_t s);
 void vec_sub(int64_t n, const double* a, const double* b, double* y, cudaStream_t s);
 // out = in - mean(in) (in == out allowed); partials: [NBLK * MAXDOT] scratch
 void vec_sub_mean(int64_t n, const double* in, double* out, double* partials, cudaStream_t s);
