@@ -188,152 +188,44 @@ __global__ void __launch_bounds__(512) k_elem_interface_b(DevMesh m, int mode, c
 
 constexpr int ELEM_THREADS = 512;
 
-// members per pass (RC) of the element kernels: 4, 8 or 16 for the 8^3 subdomains of the
-// production meshes (chosen by timing at the first ensemble call), 8 otherwise
-template <class P, int S, int RC>
+// the dense local solver's ensembles run in FP64, eight members per pass
+template <int S>
 static void elem_b_go(const DevMesh& m, bool interior, int mode, const df64* xg, const df64* in, df64* out,
                       cudaStream_t s) {
+  constexpr int RC = 8;
   const int NE = m.sx * m.sy * m.sz;
-  const size_t smem = ((size_t)m.NL * RC + (size_t)NE * 8) * sizeof(typename P::V);
+  const size_t smem = ((size_t)m.NL * RC + (size_t)NE * 8) * sizeof(double);
   if (interior) {
-    max_smem(k_elem_interior_b<P, S, RC>, smem);
-    k_elem_interior_b<P, S, RC><<<m.S, ELEM_THREADS, smem, s>>>(m, mode, xg, in, out);
+    max_smem(k_elem_interior_b<PolF64, S, RC>, smem);
+    k_elem_interior_b<PolF64, S, RC><<<m.S, ELEM_THREADS, smem, s>>>(m, mode, xg, in, out);
   } else {
-    max_smem(k_elem_interface_b<P, S, RC>, smem);
-    k_elem_interface_b<P, S, RC><<<m.S, ELEM_THREADS, smem, s>>>(m, mode, xg, in, out);
+    max_smem(k_elem_interface_b<PolF64, S, RC>, smem);
+    k_elem_interface_b<PolF64, S, RC><<<m.S, ELEM_THREADS, smem, s>>>(m, mode, xg, in, out);
   }
+  DD_CHECK_LAUNCH();
 }
 
-template <class P>
-static void elem_b_dispatch(const DevMesh& m, bool interior, int mode, const df64* xg, const df64* in,
-                            df64* out, int rc, cudaStream_t s) {
-  if (m.sx == 8 && m.sy == 8 && m.sz == 8) {
-    if (rc == 4)
-      elem_b_go<P, 8, 4>(m, interior, mode, xg, in, out, s);
-    else if (rc == 16)
-      elem_b_go<P, 8, 16>(m, interior, mode, xg, in, out, s);
-    else
-      elem_b_go<P, 8, 8>(m, interior, mode, xg, in, out, s);
-  } else if (m.sx == 4 && m.sy == 4 && m.sz == 4) {
-    elem_b_go<P, 4, 8>(m, interior, mode, xg, in, out, s);
-  } else {
-    elem_b_go<P, 0, 8>(m, interior, mode, xg, in, out, s);
-  }
-}
-
-void launch_elem_interior_b(const DevMesh& m, int mode, const df64* xg, const df64* f, df64* tI, int rc,
+static void elem_b_dispatch(const DevMesh& m, bool interior, int mode, const df64* xg, const df64* in, df64* out,
                             cudaStream_t s) {
-  if (m.schur_prec == DD_PREC_DF64)
-    elem_b_dispatch<PolDF>(m, true, mode, xg, f, tI, rc, s);
+  if (m.sx == 8 && m.sy == 8 && m.sz == 8)
+    elem_b_go<8>(m, interior, mode, xg, in, out, s);
+  else if (m.sx == 4 && m.sy == 4 && m.sz == 4)
+    elem_b_go<4>(m, interior, mode, xg, in, out, s);
   else
-    elem_b_dispatch<PolF64>(m, true, mode, xg, f, tI, 8, s);
-  DD_CHECK_LAUNCH();
+    elem_b_go<0>(m, interior, mode, xg, in, out, s);
 }
 
-void launch_elem_interface_b(const DevMesh& m, int mode, const df64* xg, const df64* sI, df64* yloc, int rc,
-                             cudaStream_t s) {
-  if (m.schur_prec == DD_PREC_DF64)
-    elem_b_dispatch<PolDF>(m, false, mode, xg, sI, yloc, rc, s);
-  else
-    elem_b_dispatch<PolF64>(m, false, mode, xg, sI, yloc, 8, s);
-  DD_CHECK_LAUNCH();
+void launch_elem_interior_b(const DevMesh& m, int mode, const df64* xg, const df64* f, df64* tI, cudaStream_t s) {
+  elem_b_dispatch(m, true, mode, xg, f, tI, s);
+}
+
+void launch_elem_interface_b(const DevMesh& m, int mode, const df64* xg, const df64* sI, df64* yloc, cudaStream_t s) {
+  elem_b_dispatch(m, false, mode, xg, sI, yloc, s);
 }
 
 // ---------------------------------------------------------------------------
-// K_II^{-1} of the ensemble: fast diagonalization with RC members per block
+// K_II^{-1} of the dense local solver
 // ---------------------------------------------------------------------------
-// contraction along axis ax, one thread per line (the other two indices and a member):
-// the line's values sit in registers and all its outputs are formed at once
-// (out_j = sum_i A(i, j) in_i when trans, else sum_i A(j, i) in_i)
-template <class P, int RC>
-__device__ __forceinline__ void fdm_contract_b(const typename P::V* A, int ax, bool trans, const int* n,
-                                               const typename P::V* in, typename P::V* out) {
-  using V = typename P::V;
-  const int na = n[ax];
-  const int stride = ax == 0 ? 1 : (ax == 1 ? n[0] : n[0] * n[1]);
-  const int o1 = ax == 0 ? n[1] : n[0];
-  const int o2 = ax == 2 ? n[1] : n[2];
-  const int nl = o1 * o2 * RC;
-  for (int t = threadIdx.x; t < nl; t += blockDim.x) {
-    const int mm = t % RC, lw = t / RC;
-    const int u = lw % o1, w = lw / o1;
-    const int base = ax == 0 ? n[0] * (u + n[1] * w) : (ax == 1 ? u + n[0] * n[1] * w : u + n[0] * w);
-    V x[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) x[i] = i < na ? in[(base + i * stride) * RC + mm] : P::zero();
-    // two outputs of the line at a time: independent accumulation chains overlap
-    const int ajs = trans ? 1 : 9, ais = trans ? 9 : 1;  // A(j, i) at A[j * ajs + i * ais]
-    for (int j = 0; j < na; j += 2) {
-      const bool two = j + 1 < na;
-      typename P::Acc a0, a1;
-      P::init(a0);
-      P::init(a1);
-#pragma unroll
-      for (int i = 0; i < 9; ++i)
-        if (i < na) {
-          P::fma(a0, A[j * ajs + i * ais], x[i]);
-          if (two) P::fma(a1, A[(j + 1) * ajs + i * ais], x[i]);
-        }
-      out[(base + j * stride) * RC + mm] = P::get(a0);
-      if (two) out[(base + (j + 1) * stride) * RC + mm] = P::get(a1);
-    }
-  }
-}
-
-// 56 lines (7 x 8: the largest two-axis face of an 8^3 subdomain's interior block) of RC
-// members per thread pass
-template <int RC>
-constexpr int fdm_threads() {
-  return 56 * RC;
-}
-
-template <class P, int RC>
-__global__ void __launch_bounds__(fdm_threads<RC>()) k_fdm_apply_b(DevMesh m, const df64* __restrict__ tI,
-                                                              df64* __restrict__ sI) {
-  using V = typename P::V;
-  extern __shared__ __align__(16) unsigned char smem_f[];
-  V* b0 = reinterpret_cast<V*>(smem_f);  // [729][RC]
-  V* b1 = b0 + 729 * RC;
-  __shared__ V Vs[3][81];
-  __shared__ int n[3];
-  const int s = blockIdx.x, m0 = blockIdx.y * RC;
-  if (threadIdx.x < 3) n[threadIdx.x] = m.fdm_n[3 * s + threadIdx.x];
-  for (int t = threadIdx.x; t < 243; t += blockDim.x) Vs[t / 81][t % 81] = ld_fdm<P>(m.fdm_V, (int64_t)s * 243 + t);
-  __syncthreads();
-  const int N = n[0] * n[1] * n[2];
-  const int64_t off = m.ioff[s];
-  for (int t = threadIdx.x; t < N * RC; t += blockDim.x)
-    b0[t] = P::from_v(tI[(off + t / RC) * BW + m0 + t % RC]);
-  __syncthreads();
-  fdm_contract_b<P, RC>(Vs[0], 0, true, n, b0, b1);
-  __syncthreads();
-  fdm_contract_b<P, RC>(Vs[1], 1, true, n, b1, b0);
-  __syncthreads();
-  fdm_contract_b<P, RC>(Vs[2], 2, true, n, b0, b1);
-  __syncthreads();
-  for (int t = threadIdx.x; t < N * RC; t += blockDim.x) {
-    typename P::Acc acc;
-    P::init(acc);
-    P::fma(acc, b1[t], ld_fdm<P>(m.fdm_Dinv, off + t / RC));
-    b1[t] = P::get(acc);
-  }
-  __syncthreads();
-  fdm_contract_b<P, RC>(Vs[0], 0, false, n, b1, b0);
-  __syncthreads();
-  fdm_contract_b<P, RC>(Vs[1], 1, false, n, b0, b1);
-  __syncthreads();
-  fdm_contract_b<P, RC>(Vs[2], 2, false, n, b1, b0);
-  __syncthreads();
-  for (int t = threadIdx.x; t < N * RC; t += blockDim.x) sI[(off + t / RC) * BW + m0 + t % RC] = P::to_v(b0[t]);
-}
-
-template <class P, int RC>
-static void fdm_b_go(const DevMesh& m, const df64* tI, df64* sI, cudaStream_t s) {
-  const size_t smem = (size_t)2 * 729 * RC * sizeof(typename P::V);
-  max_smem(k_fdm_apply_b<P, RC>, smem);
-  k_fdm_apply_b<P, RC><<<dim3(m.S, BW / RC), fdm_threads<RC>(), smem, s>>>(m, tI, sI);
-}
-
 __global__ void k_df_to_dbl(int64_t n, const df64* __restrict__ in, double* __restrict__ out) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = df64_to_double_bits(in[i]);
@@ -343,27 +235,15 @@ __global__ void k_dbl_to_df(int64_t n, const double* __restrict__ in, df64* __re
     out[i] = df64_from_double_bits(in[i]);
 }
 
-void launch_kii_apply_b(const DevMesh& m, const df64* tI, df64* sI, double* tmp, int rc, cudaStream_t s) {
-  if (m.local_solver == DD_LOCAL_FDM) {
-    if (m.schur_prec == DD_PREC_DF64) {
-      if (rc == 4)
-        fdm_b_go<PolDF, 4>(m, tI, sI, s);
-      else
-        fdm_b_go<PolDF, 8>(m, tI, sI, s);
-    } else {
-      fdm_b_go<PolF64, 8>(m, tI, sI, s);
-    }
-    DD_CHECK_LAUNCH();
-  } else {
-    // dense K_II^{-1} (FP64 tiles; the caller rejects df64 dense ensembles): the tiles work
-    // on doubles, so the block passes through tmp ([n_int][BW] doubles) both ways
-    const int64_t nn = m.n_int * BW;
-    k_df_to_dbl<<<grid_for_b(nn, 256), 256, 0, s>>>(nn, tI, tmp);
-    DD_CHECK_LAUNCH();
-    launch_symm_b(m.KIIinv, m.ioff, tmp, tmp, s);
-    k_dbl_to_df<<<grid_for_b(nn, 256), 256, 0, s>>>(nn, tmp, sI);
-    DD_CHECK_LAUNCH();
-  }
+void launch_kii_apply_b(const DevMesh& m, const df64* tI, df64* sI, double* tmp, cudaStream_t s) {
+  // FP64 tiles (the caller rejects df64 dense ensembles): the tiles work on doubles, so the
+  // block passes through tmp ([n_int][BW] doubles) both ways
+  const int64_t nn = m.n_int * BW;
+  k_df_to_dbl<<<grid_for_b(nn, 256), 256, 0, s>>>(nn, tI, tmp);
+  DD_CHECK_LAUNCH();
+  launch_symm_b(m.KIIinv, m.ioff, tmp, tmp, s);
+  k_dbl_to_df<<<grid_for_b(nn, 256), 256, 0, s>>>(nn, tmp, sI);
+  DD_CHECK_LAUNCH();
 }
 
 // ---------------------------------------------------------------------------
@@ -371,21 +251,23 @@ void launch_kii_apply_b(const DevMesh& m, const df64* tI, df64* sI, double* tmp,
 // ---------------------------------------------------------------------------
 __global__ void k_gather_b(int64_t n, const int* __restrict__ ptr, const int* __restrict__ idx,
                            const df64* __restrict__ loc, const df64* __restrict__ base,
-                           const int64_t* __restrict__ bmap, df64* __restrict__ y) {
+                           const int64_t* __restrict__ bmap, df64* __restrict__ y, int nact) {
   const int lane = threadIdx.x & 31;
+  const bool act = lane < nact;  // the local results of the padded members are not formed: zero
   for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; g < n;
        g += ((int64_t)gridDim.x * blockDim.x) >> 5) {
     // copies summed in df64 in the fixed copy order
     df64_acc sum;
     if (base) sum.add(base[(bmap ? bmap[g] : g) * BW + lane]);
-    for (int k = ptr[g]; k < ptr[g + 1]; ++k) sum.add(loc[(int64_t)idx[k] * BW + lane]);
+    if (act)
+      for (int k = ptr[g]; k < ptr[g + 1]; ++k) sum.add(loc[(int64_t)idx[k] * BW + lane]);
     y[g * BW + lane] = sum.get();
   }
 }
 void launch_gather_b(int64_t n, const int* ptr, const int* idx, const df64* loc, const df64* base,
-                     const int64_t* bmap, df64* y, cudaStream_t s) {
+                     const int64_t* bmap, df64* y, int nact, cudaStream_t s) {
   if (n == 0) return;
-  k_gather_b<<<grid_for_b(n, 8), 256, 0, s>>>(n, ptr, idx, loc, base, bmap, y);
+  k_gather_b<<<grid_for_b(n, 8), 256, 0, s>>>(n, ptr, idx, loc, base, bmap, y, nact);
   DD_CHECK_LAUNCH();
 }
 

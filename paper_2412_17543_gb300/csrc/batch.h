@@ -49,10 +49,12 @@ struct BatchWork {
   LoopCtl* ctl = nullptr;             // device-resident loop control
   LoopCtl* ctl_host = nullptr;        // pinned mirror
   double* alphas = nullptr;           // [maxit] member 0's step lengths
-  // members per pass of the element kernels and per block of the fast diagonalization
-  // (launch shapes chosen by timing at the first ensemble call), and their timings (ms)
+  int nact = BW;  // members of the current call; the local operators skip chunks of padded members
+  // members per CTA of the FDM subdomain operators (chosen by timing at the first ensemble call on
+  // 8^3 df64 subdomains), and the timings (ms); elem_rc: the element passes' members per pass, as
+  // the option asks (the FDM operators have no separate element pass)
   int elem_rc = 8, fdm_rc = 8;
-  float elem_ms[3] = {0.f, 0.f, 0.f}, fdm_ms[2] = {0.f, 0.f};
+  float fdm_ms[2] = {0.f, 0.f};
   // symmetric products of the ensemble (level-1 N_i; level-2 K_II^{-1} and N): tensor-core
   // operand copy, the kernel in use, and the selection timings (SIMT, 3xTF32, BF16x3)
   struct SymOp {
@@ -71,16 +73,13 @@ void launch_pack_out(int64_t n, int nrhs, const df64* in, double* X, cudaStream_
 void launch_to_float(int64_t n, const double* in, float* out, cudaStream_t s);
 
 // ---- Schur-complement operator (interleaved counterparts of the single-vector kernels) ----
-// rc: members per pass of the element kernels (4, 8 or 16; used for 8^3 subdomains, df64)
-void launch_elem_interior_b(const DevMesh& m, int mode, const df64* xg, const df64* f, df64* tI, int rc,
-                            cudaStream_t s);
-void launch_elem_interface_b(const DevMesh& m, int mode, const df64* xg, const df64* sI, df64* yloc, int rc,
-                             cudaStream_t s);
-// tmp: [n_int][BW] doubles, used by the dense local solver only; rc: members per block of
-// the fast diagonalization (4 or 8, df64)
-void launch_kii_apply_b(const DevMesh& m, const df64* tI, df64* sI, double* tmp, int rc, cudaStream_t s);
+// element passes and K_II^{-1} of the dense local solver (FP64); tmp: [n_int][BW] doubles
+void launch_elem_interior_b(const DevMesh& m, int mode, const df64* xg, const df64* f, df64* tI, cudaStream_t s);
+void launch_elem_interface_b(const DevMesh& m, int mode, const df64* xg, const df64* sI, df64* yloc, cudaStream_t s);
+void launch_kii_apply_b(const DevMesh& m, const df64* tI, df64* sI, double* tmp, cudaStream_t s);
+// y[g] = base + sum of the copies of loc (members below nact; the others' copies count as zero)
 void launch_gather_b(int64_t n, const int* ptr, const int* idx, const df64* loc, const df64* base,
-                     const int64_t* bmap, df64* y, cudaStream_t s);
+                     const int64_t* bmap, df64* y, int nact, cudaStream_t s);
 void launch_scatter_recover_b(const DevMesh& m, const df64* xg, const df64* sI, df64* x, cudaStream_t s);
 
 // ---- BDDC (T = float or double by prec) ----

@@ -85,6 +85,18 @@ struct BatchedRows {
   unsigned* zticket = nullptr;    // [count][column blocks] counters, 0 between launches
 };
 
+// Assembled rows of the local stiffness matrices that touch the interface (see local.h).
+struct LocalRows {
+  const int* type = nullptr;
+  const int* trange = nullptr;
+  const int* sl_off = nullptr;
+  const int16_t *sl_out = nullptr, *sl_cnt = nullptr, *nb = nullptr;
+  const int64_t* coff = nullptr;
+  const void* coef = nullptr;   // df64 or double, as schur_prec
+  const int* ifree = nullptr;   // [n_int] free node of each interior unknown
+  int max_loc = 0;              // largest local vector (interface and interior)
+};
+
 // Level-1 geometry and Schur-complement operator (Sect. 3.1).
 struct DevMesh {
   int nx, ny, nz, sx, sy, sz, Sx, Sy, Sz, S;
@@ -117,8 +129,9 @@ struct DevMesh {
   const int* fdm_n;         // [S][3] sizes of the interior index sets per axis (<= 9)
   const void* fdm_V;        // [S][3][81] 1D generalized eigenvectors, stride 9 (df64 or double)
   const void* fdm_Dinv;     // [n_int] inverse eigenvalue sums, indexed like interior vectors
+  LocalRows rows;           // local_solver == DD_LOCAL_FDM
   // per-subdomain copies read by the fused Schur kernel in one coalesced level each
-  // (8^3-element subdomains with the fast-diagonalization solver only; else null):
+  // (df64 operator on 8^3-element subdomains with the fast-diagonalization solver only; else null):
   const int* sxg = nullptr;     // [S][NL] interface index of each local node (-1: not on the interface)
   const void* sfac = nullptr;   // [S][max_nbl][3] factors of the boundary-layer elements in the
                                 // order of the type's list (df64 or double, as schur_prec)
@@ -169,8 +182,8 @@ constexpr int COARSE_DENSE_MAX_B = 2048;  // ensembles: each block of 8 rows rea
 
 // Scratch buffers of the operators (device).
 struct Work {
-  double* tI;      // [n_int] level-1 interior
-  double* sI;      // [n_int]
+  double* tI = nullptr;  // [n_int] level-1 interior (dense local solver)
+  double* sI = nullptr;  // [n_int]
   double* yloc;    // [n_flat] level-1 local interface
   double* rloc;    // [n_flat]
   double* uloc;    // [n_flat]
@@ -197,12 +210,11 @@ struct Work {
 enum ElemMode { ELEM_SCHUR = 0, ELEM_CONDENSE = 1, ELEM_RECOVER = 2 };
 
 // ---- launch wrappers (kernels.cu) ----
+// element passes of the dense local solver
 void launch_elem_interior(const DevMesh& m, int mode, const double* xg, const double* f, double* tI, cudaStream_t s);
 void launch_elem_interface(const DevMesh& m, int mode, const double* xg, const double* sI, double* yloc,
                            cudaStream_t s);
-// s_I = K_II^{-1} t_I for every subdomain (dense tiles or fast diagonalization)
-void launch_kii_apply(const DevMesh& m, const double* tI, double* sI, int* err, cudaStream_t s);
-// fused Schur application (one CTA per subdomain) for the fast-diagonalization solver of 8^3 subdomains
+// fused Schur application (one CTA per subdomain), df64 on 8^3 subdomains with the FDM solver
 bool schur_fused_available(const DevMesh& m);
 void launch_schur_fused(const DevMesh& m, const double* xg, double* yloc, cudaStream_t s);
 void launch_symv(const SymTiles& A, const int64_t* voff, const double* in, double* out, int* err, cudaStream_t s);

@@ -16,6 +16,7 @@
 
 #include "batch.h"
 #include "context.h"
+#include "local.h"
 
 namespace dd {
 
@@ -101,38 +102,23 @@ void select_op(dd_ctx* c, int which, const SymTiles& S, const int64_t* voff, voi
 }
 
 
-// launch shapes of the Schur operator of the ensemble: members per pass of the element
-// kernels (4, 8, 16) and per block of the fast diagonalization (4, 8), taken from the
-// options or else each timed on the context's own mesh (df64 operator on 8^3 subdomains;
-// other meshes keep 8)
+// members per CTA of the Schur operator of the ensemble (4 or 8): from the options or else timed on
+// the context's own mesh (df64 operator on 8^3 subdomains; other meshes keep 8)
 void select_shapes(dd_ctx* c, cudaStream_t s) {
   BatchWork& B = *c->bw;
   const DevMesh& m = c->mesh;
   if (m.schur_prec != DD_PREC_DF64 || !(m.sx == 8 && m.sy == 8 && m.sz == 8)) return;
-  const int64_t n = c->n_gamma;
-  DD_CUDA(cudaMemsetAsync(B.p, 0, (size_t)n * BW * sizeof(df64), s));
-  DD_CUDA(cudaMemsetAsync(B.sI, 0, (size_t)std::max<int64_t>(m.n_int, 1) * BW * sizeof(df64), s));
-  if (c->opt.ens_elem_rc) {
-    B.elem_rc = c->opt.ens_elem_rc;
-  } else {
-    const int rcs[3] = {4, 8, 16};
-    int best = 1;
-    for (int v = 0; v < 3; ++v) {
-      B.elem_ms[v] = time_ms([&] { launch_elem_interface_b(m, ELEM_SCHUR, B.p, B.sI, B.yloc, rcs[v], s); }, s);
-      if (B.elem_ms[v] < B.elem_ms[best]) best = v;
-    }
-    B.elem_rc = rcs[best];
+  if (c->opt.ens_elem_rc) B.elem_rc = c->opt.ens_elem_rc;
+  if (m.local_solver != DD_LOCAL_FDM) return;
+  if (c->opt.ens_fdm_rc) {
+    B.fdm_rc = c->opt.ens_fdm_rc;
+    return;
   }
-  if (m.local_solver == DD_LOCAL_FDM) {
-    if (c->opt.ens_fdm_rc) {
-      B.fdm_rc = c->opt.ens_fdm_rc;
-    } else {
-      for (int v = 0; v < 2; ++v)
-        B.fdm_ms[v] = time_ms([&] { launch_kii_apply_b(m, B.sI, B.tI, B.kii_tmp, v == 0 ? 4 : 8, s); }, s);
-      B.fdm_rc = B.fdm_ms[0] < B.fdm_ms[1] ? 4 : 8;
-    }
-  }
-  check_err(c, s);
+  DD_CUDA(cudaMemsetAsync(B.p, 0, (size_t)c->n_gamma * BW * sizeof(df64), s));
+  for (int v = 0; v < 2; ++v)
+    B.fdm_ms[v] =
+        time_ms([&] { launch_local_apply_b(m, ELEM_SCHUR, v == 0 ? 4 : 8, BW, B.p, nullptr, B.yloc, s); }, s);
+  B.fdm_rc = B.fdm_ms[0] < B.fdm_ms[1] ? 4 : 8;
 }
 
 // whether the ensemble applies the level-2 BDDC as the explicit matrix
@@ -188,8 +174,10 @@ BatchWork& batch_work(dd_ctx* c, cudaStream_t s) {
   const int64_t n = c->n_gamma;
   auto dvec = [&](int64_t rows) { return A.alloc<df64>((size_t)std::max<int64_t>(rows, 1) * BW); };
   auto tvec = [&](int prec, int64_t rows) { return typed_vec(A, prec, rows); };
-  B->tI = dvec(m.n_int);
-  B->sI = dvec(m.n_int);
+  if (m.local_solver != DD_LOCAL_FDM) {
+    B->tI = dvec(m.n_int);
+    B->sI = dvec(m.n_int);
+  }
   B->yloc = dvec(c->b1.n_flat);
   if (m.local_solver != DD_LOCAL_FDM) B->kii_tmp = A.alloc<double>((size_t)std::max<int64_t>(m.n_int, 1) * BW);
   B->D1f = A.alloc<float>((size_t)std::max<int64_t>(c->b1.n_flat, 1));
@@ -230,24 +218,36 @@ BatchWork& batch_work(dd_ctx* c, cudaStream_t s) {
 void schur_b(dd_ctx* c, const df64* x, df64* y, cudaStream_t s) {
   ProfScope ps(c, DD_PROF_ENS_SCHUR, s);
   BatchWork& B = *c->bw;
-  launch_elem_interior_b(c->mesh, ELEM_SCHUR, x, nullptr, B.tI, B.elem_rc, s);
-  launch_kii_apply_b(c->mesh, B.tI, B.sI, B.kii_tmp, B.fdm_rc, s);
-  launch_elem_interface_b(c->mesh, ELEM_SCHUR, x, B.sI, B.yloc, B.elem_rc, s);
-  launch_gather_b(c->n_gamma, c->mesh.gptr, c->mesh.gidx, B.yloc, nullptr, nullptr, y, s);
+  if (c->mesh.local_solver == DD_LOCAL_FDM) {
+    launch_local_apply_b(c->mesh, ELEM_SCHUR, B.fdm_rc, B.nact, x, nullptr, B.yloc, s);
+  } else {
+    launch_elem_interior_b(c->mesh, ELEM_SCHUR, x, nullptr, B.tI, s);
+    launch_kii_apply_b(c->mesh, B.tI, B.sI, B.kii_tmp, s);
+    launch_elem_interface_b(c->mesh, ELEM_SCHUR, x, B.sI, B.yloc, s);
+  }
+  launch_gather_b(c->n_gamma, c->mesh.gptr, c->mesh.gidx, B.yloc, nullptr, nullptr, y, B.nact, s);
 }
 
 void condense_b(dd_ctx* c, const df64* f, df64* b, cudaStream_t s) {
   BatchWork& B = *c->bw;
-  launch_elem_interior_b(c->mesh, ELEM_CONDENSE, nullptr, f, B.tI, B.elem_rc, s);
-  launch_kii_apply_b(c->mesh, B.tI, B.sI, B.kii_tmp, B.fdm_rc, s);
-  launch_elem_interface_b(c->mesh, ELEM_CONDENSE, nullptr, B.sI, B.yloc, B.elem_rc, s);
-  launch_gather_b(c->n_gamma, c->mesh.gptr, c->mesh.gidx, B.yloc, f, c->mesh.gamma_free, b, s);
+  if (c->mesh.local_solver == DD_LOCAL_FDM) {
+    launch_local_apply_b(c->mesh, ELEM_CONDENSE, B.fdm_rc, B.nact, nullptr, f, B.yloc, s);
+  } else {
+    launch_elem_interior_b(c->mesh, ELEM_CONDENSE, nullptr, f, B.tI, s);
+    launch_kii_apply_b(c->mesh, B.tI, B.sI, B.kii_tmp, s);
+    launch_elem_interface_b(c->mesh, ELEM_CONDENSE, nullptr, B.sI, B.yloc, s);
+  }
+  launch_gather_b(c->n_gamma, c->mesh.gptr, c->mesh.gidx, B.yloc, f, c->mesh.gamma_free, b, B.nact, s);
 }
 
 void recover_b(dd_ctx* c, const df64* f, const df64* xg, df64* x, cudaStream_t s) {
   BatchWork& B = *c->bw;
-  launch_elem_interior_b(c->mesh, ELEM_RECOVER, xg, f, B.tI, B.elem_rc, s);
-  launch_kii_apply_b(c->mesh, B.tI, B.sI, B.kii_tmp, B.fdm_rc, s);
+  if (c->mesh.local_solver == DD_LOCAL_FDM) {
+    launch_local_apply_b(c->mesh, ELEM_RECOVER, B.fdm_rc, B.nact, xg, f, x, s);
+    return;
+  }
+  launch_elem_interior_b(c->mesh, ELEM_RECOVER, xg, f, B.tI, s);
+  launch_kii_apply_b(c->mesh, B.tI, B.sI, B.kii_tmp, s);
   launch_scatter_recover_b(c->mesh, xg, B.sI, x, s);
 }
 
@@ -404,6 +404,7 @@ dd_status pcg_solve_b(dd_ctx* c, dd_recycle* st, double rtol, bool record, int n
                                      (uint64_t)rec,
                                      (uint64_t)st->hmax,
                                      (uint64_t)flex,
+                                     (uint64_t)B.nact,
                                      (uint64_t)(uintptr_t)W,
                                      (uint64_t)(uintptr_t)AW,
                                      (uint64_t)(uintptr_t)st->Ginv,
@@ -498,6 +499,7 @@ static dd_status batch_op(dd_ctx* c, int32_t nrhs, const double* X, double* Y, v
   return guard_call([&] {
     cudaStream_t s = (cudaStream_t)stream;
     BatchWork& B = batch_work(c, s);
+    B.nact = nrhs;
     launch_pack_in(c->n_gamma, nrhs, X, B.p, s);
     if (precond)
       precond_b(c, B.p, B.q, s);
@@ -535,6 +537,7 @@ dd_status dd_solve_batch(dd_ctx* c, int32_t nrhs, const double* F, double* X, do
     cudaStream_t s = (cudaStream_t)stream;
     BatchWork& B = batch_work(c, s);
     DD_CUDA(cudaEventRecord(c->ev0, s));
+    B.nact = nrhs;
     launch_pack_in(c->n_free, nrhs, F, B.F, s);
     condense_b(c, B.F, B.bvec, s);
     copy_b(B.xg, st->xg_prev_b, c->n_gamma, s);

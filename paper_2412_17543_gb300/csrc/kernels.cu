@@ -608,75 +608,14 @@ void launch_wait_selftest(int* err, long long limit, cudaStream_t s) {
 
 
 // ---------------------------------------------------------------------------
-// Fast diagonalization: s = V D^{-1} V^T t with V = Vz (x) Vy (x) Vx, one CTA per subdomain,
-// six contractions along one axis each in shared memory (about 14k multiply-adds per
-// 8^3 subdomain instead of a 343^2 matrix).
-// ---------------------------------------------------------------------------
-// out[..j..] = sum_i A(i, j) in[..i..] (transposed) or sum_i A(j, i) in[..i..] along axis `ax`
-template <class P>
-__device__ __forceinline__ void fdm_contract(const typename P::V* A, int ax, bool trans, const int* n,
-                                             const typename P::V* in, typename P::V* out) {
-  const int N = n[0] * n[1] * n[2];
-  const int na = n[ax];
-  const int stride = ax == 0 ? 1 : (ax == 1 ? n[0] : n[0] * n[1]);
-  for (int idx = threadIdx.x; idx < N; idx += blockDim.x) {
-    const int j = (idx / stride) % na;
-    const int base = idx - j * stride;
-    typename P::Acc acc[2];
-    P::init(acc[0]);
-    P::init(acc[1]);
-    for (int i = 0; i < na; ++i) {
-      typename P::V a = trans ? A[i * 9 + j] : A[j * 9 + i];
-      P::fma(acc[i & 1], a, in[base + i * stride]);
-    }
-    out[idx] = P::add(P::get(acc[0]), P::get(acc[1]));
-  }
-}
-
-template <class P>
-__global__ void __launch_bounds__(128) k_fdm_apply(DevMesh m, const double* __restrict__ tI, double* __restrict__ sI) {
-  using V = typename P::V;
-  __shared__ V Vs[3][81];
-  __shared__ V b0[729], b1[729];
-  __shared__ int n[3];
-  const int s = blockIdx.x;
-  if (threadIdx.x < 3) n[threadIdx.x] = m.fdm_n[3 * s + threadIdx.x];
-  for (int t = threadIdx.x; t < 243; t += blockDim.x) Vs[t / 81][t % 81] = ld_fdm<P>(m.fdm_V, (int64_t)s * 243 + t);
-  __syncthreads();
-  const int N = n[0] * n[1] * n[2];
-  const int64_t off = m.ioff[s];
-  for (int i = threadIdx.x; i < N; i += blockDim.x) b0[i] = P::from_d(tI[off + i]);
-  __syncthreads();
-  fdm_contract<P>(Vs[0], 0, true, n, b0, b1);
-  __syncthreads();
-  fdm_contract<P>(Vs[1], 1, true, n, b1, b0);
-  __syncthreads();
-  fdm_contract<P>(Vs[2], 2, true, n, b0, b1);
-  __syncthreads();
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    typename P::Acc acc;
-    P::init(acc);
-    P::fma(acc, b1[i], ld_fdm<P>(m.fdm_Dinv, off + i));
-    b1[i] = P::get(acc);
-  }
-  __syncthreads();
-  fdm_contract<P>(Vs[0], 0, false, n, b1, b0);
-  __syncthreads();
-  fdm_contract<P>(Vs[1], 1, false, n, b0, b1);
-  __syncthreads();
-  fdm_contract<P>(Vs[2], 2, false, n, b1, b0);
-  __syncthreads();
-  for (int i = threadIdx.x; i < N; i += blockDim.x) sI[off + i] = P::to_d(b0[i]);
-}
-
-// ---------------------------------------------------------------------------
 // Fused Schur-complement application y_i = (K_GG - K_GI K_II^{-1} K_IG) x_i of one
 // subdomain per CTA (eq. 6) for the fast-diagonalization local solver: the interior pass
 // (t_I = K_IG x_G), the six contractions of K_II^{-1} and the interface pass
 // (y_G = K_GG x_G - K_GI s_I) run back to back on shared memory, so the interior
 // vectors never leave the SM and the element entries of the boundary-layer elements
-// are formed once. The arithmetic and its order are those of k_elem_interior,
-// k_fdm_apply and k_elem_interface.
+// are formed once. Single vectors in df64 on 8^3 subdomains only: the assembled rows of local.cu, which
+// serve every other case, stream 77 KB of coefficients per subdomain and were slower for these (128^3:
+// 0.194 against 0.168 ms; in the 64^3 loop, with the coefficients cold, 3.95 against 3.70 ms a solve).
 // ---------------------------------------------------------------------------
 // The same contractions with an epilogue: EPI 0 stores out[idx], EPI 1 stores
 // out[idx] * dv[idx] (the diagonal D^{-1} of the fast diagonalization), EPI 2 stores
@@ -871,7 +810,7 @@ __global__ void __launch_bounds__(BS) k_schur_fused(DevMesh m, const double* __r
 }
 
 bool schur_fused_available(const DevMesh& m) {
-  return m.local_solver == DD_LOCAL_FDM && m.sx == 8 && m.sy == 8 && m.sz == 8 && m.type_citems != nullptr &&
+  return m.schur_prec == DD_PREC_DF64 && m.local_solver == DD_LOCAL_FDM && m.sx == 8 && m.sy == 8 && m.sz == 8 && m.type_citems != nullptr &&
          m.sxg != nullptr && m.sfac != nullptr && m.max_nint > 0 && m.max_nint <= m.NL;
 }
 
@@ -882,37 +821,17 @@ static void schur_fused_bs(const DevMesh& m, const double* xg, double* yloc, siz
 }
 
 void launch_schur_fused(const DevMesh& m, const double* xg, double* yloc, cudaStream_t s) {
-  const size_t vb = m.schur_prec == DD_PREC_DF64 ? sizeof(df64) : sizeof(double);
+  const size_t vb = sizeof(df64);
   // interior buffers sized by the largest interior of a subdomain (up to 8^3 on the Neumann
   // boundary, whose face nodes are interior unknowns), so that more CTAs fit on an SM
   const size_t ni = (size_t)m.max_nint;
   const size_t smem = vb * ((size_t)m.NL + 3 * ni + 243 + 8 * (size_t)m.max_nbl) + 2 * ((size_t)m.max_nbl + ni);
-  if (m.schur_prec == DD_PREC_DF64) {
-    switch (m.schur_threads) {
-      case 352: schur_fused_bs<PolDF, 352>(m, xg, yloc, smem, s); break;
-      case 416: schur_fused_bs<PolDF, 416>(m, xg, yloc, smem, s); break;
-      default: schur_fused_bs<PolDF, 256>(m, xg, yloc, smem, s);
-    }
-  } else {
-    switch (m.schur_threads) {
-      case 352: schur_fused_bs<PolF64, 352>(m, xg, yloc, smem, s); break;
-      case 416: schur_fused_bs<PolF64, 416>(m, xg, yloc, smem, s); break;
-      default: schur_fused_bs<PolF64, 256>(m, xg, yloc, smem, s);
-    }
+  switch (m.schur_threads) {
+    case 352: schur_fused_bs<PolDF, 352>(m, xg, yloc, smem, s); break;
+    case 416: schur_fused_bs<PolDF, 416>(m, xg, yloc, smem, s); break;
+    default: schur_fused_bs<PolDF, 256>(m, xg, yloc, smem, s);
   }
   DD_CHECK_LAUNCH();
-}
-
-void launch_kii_apply(const DevMesh& m, const double* tI, double* sI, int* err, cudaStream_t s) {
-  if (m.local_solver == DD_LOCAL_FDM) {
-    if (m.schur_prec == DD_PREC_DF64)
-      k_fdm_apply<PolDF><<<m.S, 128, 0, s>>>(m, tI, sI);
-    else
-      k_fdm_apply<PolF64><<<m.S, 128, 0, s>>>(m, tI, sI);
-    DD_CHECK_LAUNCH();
-  } else {
-    launch_symv(m.KIIinv, m.ioff, tI, sI, err, s);
-  }
 }
 
 // ---------------------------------------------------------------------------

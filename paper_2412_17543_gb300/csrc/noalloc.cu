@@ -8,6 +8,7 @@
 
 #include "common.h"
 #include "device.h"
+#include "local.h"
 
 namespace dd {
 const DevMesh* context_mesh(const dd_ctx* c);
@@ -66,9 +67,15 @@ extern "C" dd_status dd_schur_apply_noalloc(dd_ctx* ctx, const double* x, double
     // stream-ordered launches only: the call returns without waiting for the GPU. A bounded
     // wait that gives up in these kernels sets the context's error word, which the next
     // entry point of the context that reads it reports as DD_TIMEOUT.
-    dd::launch_elem_interior(m, dd::ELEM_SCHUR, x, nullptr, tI, s);
-    dd::launch_kii_apply(m, tI, sI, dd::context_err(ctx), s);
-    dd::launch_elem_interface(m, dd::ELEM_SCHUR, x, sI, yloc, s);
+    if (dd::schur_fused_available(m)) {
+      dd::launch_schur_fused(m, x, yloc, s);
+    } else if (m.local_solver == DD_LOCAL_FDM) {
+      dd::launch_local_apply(m, dd::ELEM_SCHUR, x, nullptr, yloc, s);
+    } else {
+      dd::launch_elem_interior(m, dd::ELEM_SCHUR, x, nullptr, tI, s);
+      dd::launch_symv(m.KIIinv, m.ioff, tI, sI, dd::context_err(ctx), s);
+      dd::launch_elem_interface(m, dd::ELEM_SCHUR, x, sI, yloc, s);
+    }
     dd::launch_gather(m.n_gamma, m.gptr, m.gidx, yloc, nullptr, nullptr, y, s);
     return DD_OK;
   } catch (const dd::Error& err) {

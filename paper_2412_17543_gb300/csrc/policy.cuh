@@ -25,6 +25,7 @@ struct PolF64 {
   __device__ static void init(Acc& a) { a = 0.0; }
   __device__ static void fma(Acc& a, V k, V x) { a = ::fma(k, x, a); }
   __device__ static V get(const Acc& a) { return a; }
+  __device__ static void merge(Acc& a, const Acc& b) { a += b; }
   __device__ static V add(V a, V b) { return a + b; }
   // element entry for corner pair differing on axes d (bit0 x, bit1 y, bit2 z)
   __device__ static V entry(const V* c, int d) {
@@ -47,6 +48,7 @@ struct PolDF {
   __device__ static void init(Acc& a) { a = df64_acc(); }
   __device__ static void fma(Acc& a, V k, V x) { a.fma(k, x); }
   __device__ static V get(const Acc& a) { return a.get(); }
+  __device__ static void merge(Acc& a, const Acc& b) { a.add(df64{b.s, b.c}); }  // a += b, error-free in the leading parts
   __device__ static V add(V a, V b) { return df64_add(a, b); }
   __device__ static V entry(const V* c, int d) {
     // the scalings are +-1, +-2, +-4: exact on both halves

@@ -20,6 +20,7 @@
 #include "setup.h"
 #include "vecops.h"
 #include "context.h"
+#include "local.h"
 #include "batch.h"
 #include "recycle.h"
 
@@ -219,10 +220,14 @@ void schur_local(dd_ctx* c, const double* x, cudaStream_t s) {
     launch_schur_fused(c->mesh, x, c->w.yloc, s);
     return;
   }
+  if (c->mesh.local_solver == DD_LOCAL_FDM) {
+    launch_local_apply(c->mesh, ELEM_SCHUR, x, nullptr, c->w.yloc, s);
+    return;
+  }
   launch_elem_interior(c->mesh, ELEM_SCHUR, x, nullptr, c->w.tI, s);
   {
     ProfScope pk(c, DD_PROF_SYMV_KII, s);
-    launch_kii_apply(c->mesh, c->w.tI, c->w.sI, c->w.err, s);
+    launch_symv(c->mesh.KIIinv, c->mesh.ioff, c->w.tI, c->w.sI, c->w.err, s);
   }
   launch_elem_interface(c->mesh, ELEM_SCHUR, x, c->w.sI, c->w.yloc, s);
 }
@@ -234,15 +239,23 @@ void schur_apply(dd_ctx* c, const double* x, double* y, cudaStream_t s) {
 }
 
 void condense(dd_ctx* c, const double* f, double* b, cudaStream_t s) {
-  launch_elem_interior(c->mesh, ELEM_CONDENSE, nullptr, f, c->w.tI, s);
-  launch_kii_apply(c->mesh, c->w.tI, c->w.sI, c->w.err, s);
-  launch_elem_interface(c->mesh, ELEM_CONDENSE, nullptr, c->w.sI, c->w.yloc, s);
+  if (c->mesh.local_solver == DD_LOCAL_FDM) {
+    launch_local_apply(c->mesh, ELEM_CONDENSE, nullptr, f, c->w.yloc, s);
+  } else {
+    launch_elem_interior(c->mesh, ELEM_CONDENSE, nullptr, f, c->w.tI, s);
+    launch_symv(c->mesh.KIIinv, c->mesh.ioff, c->w.tI, c->w.sI, c->w.err, s);
+    launch_elem_interface(c->mesh, ELEM_CONDENSE, nullptr, c->w.sI, c->w.yloc, s);
+  }
   launch_gather(c->n_gamma, c->mesh.gptr, c->mesh.gidx, c->w.yloc, f, c->mesh.gamma_free, b, s);
 }
 
 void recover(dd_ctx* c, const double* f, const double* xg, double* x, cudaStream_t s) {
+  if (c->mesh.local_solver == DD_LOCAL_FDM) {
+    launch_local_apply(c->mesh, ELEM_RECOVER, xg, f, x, s);
+    return;
+  }
   launch_elem_interior(c->mesh, ELEM_RECOVER, xg, f, c->w.tI, s);
-  launch_kii_apply(c->mesh, c->w.tI, c->w.sI, c->w.err, s);
+  launch_symv(c->mesh.KIIinv, c->mesh.ioff, c->w.tI, c->w.sI, c->w.err, s);
   launch_scatter_recover(c->mesh, xg, c->w.sI, x, s);
 }
 
@@ -501,7 +514,7 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
   Work& w = c->w;
   DD_CUDA(cudaMemsetAsync(c->r, 0, c->n_gamma * sizeof(double), s));
   DD_CUDA(cudaMemsetAsync(w.rloc, 0, c->b1.n_flat * sizeof(double), s));
-  DD_CUDA(cudaMemsetAsync(w.tI, 0, c->mesh.n_int * sizeof(double), s));
+  if (w.tI) DD_CUDA(cudaMemsetAsync(w.tI, 0, c->mesh.n_int * sizeof(double), s));
   DD_CUDA(cudaMemsetAsync(c->p, 0, c->n_gamma * sizeof(double), s));
   auto tune_sym = [&](SymTiles& A, const int64_t* voff, const double* in, double* out, float* ms) {
     if (A.count < 152) return;  // a small batch leaves most SMs idle whatever the ring depth
@@ -686,6 +699,7 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
     DevMesh& dm = c->mesh;
     std::vector<double> elem_madds, elem_nbl;  // per subdomain type (for the profiling counts)
     std::vector<int> elem_type;
+    std::vector<double> rows_madds;  // per subdomain: stored row entries (FDM)
     dm.nx = M.nx; dm.ny = M.ny; dm.nz = M.nz; dm.sx = M.sx; dm.sy = M.sy; dm.sz = M.sz;
     dm.Sx = M.Sx; dm.Sy = M.Sy; dm.Sz = M.Sz; dm.S = M.S;
     dm.fx0 = M.fx0; dm.fx1 = M.fx1; dm.fy0 = M.fy0; dm.fy1 = M.fy1; dm.fz0 = M.fz0; dm.fz1 = M.fz1;
@@ -719,7 +733,7 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
       for (int i = 0; i < M.S; ++i)
         dm.max_nint = std::max(dm.max_nint, (int)(H->l1.ioff[i + 1] - H->l1.ioff[i]));
       dm.schur_threads = 256;
-      if (H->local_solver == DD_LOCAL_FDM && M.sx == 8 && M.sy == 8 && M.sz == 8) {
+      if (opt->schur_prec == DD_PREC_DF64 && H->local_solver == DD_LOCAL_FDM && M.sx == 8 && M.sy == 8 && M.sz == 8) {
         // the fused Schur kernel's per-subdomain copies: each local node's interface index, and
         // the factors of the boundary-layer elements in the order of the type's list
         std::vector<int> sxg((size_t)M.S * M.NL, -1);
@@ -741,13 +755,9 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
           }
         }
         dm.sxg = A.upload(sxg, s);
-        if (opt->schur_prec == DD_PREC_DF64) {
-          std::vector<df64> sfd(sf.size());
-          for (size_t t = 0; t < sf.size(); ++t) sfd[t] = df64_from_double(sf[t]);
-          dm.sfac = A.upload(sfd, s);
-        } else {
-          dm.sfac = A.upload(sf, s);
-        }
+        std::vector<df64> sfd(sf.size());
+        for (size_t t = 0; t < sf.size(); ++t) sfd[t] = df64_from_double(sf[t]);
+        dm.sfac = A.upload(sfd, s);
       }
     }
     dm.ioff = A.upload(H->l1.ioff, s);
@@ -795,6 +805,40 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
         dm.fdm_V = A.upload(Vd, s);
         dm.fdm_Dinv = A.upload(Dd, s);
       }
+      const LocalRowsHost R = build_local_rows(M, H->l1);
+      LocalRows& lr = dm.rows;
+      lr.type = A.upload(R.type, s);
+      lr.trange = A.upload(R.trange, s);
+      lr.sl_off = A.upload(R.sl_off, s);
+      lr.sl_out = A.upload(R.sl_out, s);
+      lr.sl_cnt = A.upload(R.sl_cnt, s);
+      lr.nb = A.upload(R.nb, s);
+      lr.coff = A.upload(R.coff, s);
+      if (opt->schur_prec == DD_PREC_DF64) {
+        std::vector<df64> cf(R.coef.size());
+#pragma omp parallel for schedule(static)
+        for (int64_t t = 0; t < (int64_t)cf.size(); ++t) cf[t] = df64_from_double(R.coef[t]);
+        lr.coef = A.upload(cf, s);
+      } else {
+        lr.coef = A.upload(R.coef, s);
+      }
+      std::vector<int> ifree((size_t)dm.n_int);
+      const int64_t Nfx = M.fx1 - M.fx0, Nfy = M.fy1 - M.fy0;
+      for (int i = 0; i < M.S; ++i) {
+        const int16_t* code = M.lidx.data() + (size_t)i * M.NL;
+        const int I = i % M.Sx, J = (i / M.Sx) % M.Sy, K = i / (M.Sx * M.Sy);
+        for (int l = 0; l < M.NL; ++l)
+          if (code[l] >= 0) {
+            const int a = l % M.NLx, b = (l / M.NLx) % M.NLy, q = l / (M.NLx * M.NLy);
+            ifree[H->l1.ioff[i] + code[l]] = (int)((I * M.sx + a - M.fx0) +
+                                                   Nfx * ((J * M.sy + b - M.fy0) + Nfy * (int64_t)(K * M.sz + q - M.fz0)));
+          }
+        lr.max_loc = std::max(lr.max_loc, (int)(H->l1.ioff[i + 1] - H->l1.ioff[i] + H->l1.goff[i + 1] - H->l1.goff[i]));
+      }
+      lr.ifree = A.upload(ifree, s);
+      // multiply-adds and element data of the profile: the rows' entries
+      rows_madds.resize(M.S);
+      for (int i = 0; i < M.S; ++i) rows_madds[i] = (double)(R.coff[i + 1] - R.coff[i]);
       dm.KIIinv.count = 0;
     } else {
       std::vector<const double*> mats;
@@ -809,8 +853,10 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
     upload_bddc(A, H->l1, opt->precond_prec, c->b1, s);
     int pp = opt->precond_prec;
     Work& w = c->w;
-    w.tI = A.alloc<double>(dm.n_int);
-    w.sI = A.alloc<double>(dm.n_int);
+    if (H->local_solver != DD_LOCAL_FDM) {
+      w.tI = A.alloc<double>(dm.n_int);
+      w.sI = A.alloc<double>(dm.n_int);
+    }
     w.yloc = A.alloc<double>(c->b1.n_flat);
     w.rloc = A.alloc<double>(c->b1.n_flat);
     w.uloc = A.alloc<double>(c->b1.n_flat);
@@ -921,8 +967,9 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
       const double n_flat = (double)H->l1.goff[M.S], n_g = (double)c->n_gamma;
       for (int i = 0; i < M.S; ++i) {
         const int t = elem_type[i];
-        sm += elem_madds[t];
-        sb += elem_nbl[t] * 3 * 8.0 + M.NL * 2.0;
+        const bool rows = H->local_solver == DD_LOCAL_FDM && !schur_fused_available(dm);
+        sm += rows ? rows_madds[i] : elem_madds[t];
+        sb += rows ? rows_madds[i] * 8.0 : elem_nbl[t] * 3 * 8.0 + M.NL * 2.0;
         const double a = H->l1.sub[i].nI;
         if (H->local_solver == DD_LOCAL_FDM) {
           const FdmSub& F = H->fdm[i];
