@@ -350,24 +350,49 @@ __device__ __forceinline__ typename P::V packed_diag_part(const unsigned char* T
 }
 
 // block of the ragged last w columns (32 rows of wp stored values): lane l returns the row
-// part sum_{c<w} T(l, c) x_j[c] and, for l < w, the column part sum_r T(r, l) x_i[r]
+// part sum_{c<w} T(l, c) x_j[c] and, for l < w, the column part sum_r T(r, l) x_i[r].
+// A few columns: one warp sum each. More: the lanes walk their rows from different columns
+// (c = l mod w onwards, so that their shared-memory addresses spread over the banks) and their columns
+// down the rows, both without shuffles. The warp sums cost about 300 cycles a column in df64: with
+// 23 of 32 columns (n = 343) the ten ragged blocks took as long as the 45 full ones.
 template <class P>
 __device__ __forceinline__ void packed_ragged_parts(const unsigned char* T, int wp, int w, const typename P::V* ti,
                                                     const typename P::V* tj, int l, typename P::V& row,
                                                     typename P::V& col) {
-  typename P::Acc ar;
-  P::init(ar);
+  typename P::Acc ar[2];
+  P::init(ar[0]);
+  P::init(ar[1]);
   col = P::zero();
-  for (int c = 0; c < w; ++c) {
-    const typename P::V e = TileElem<P>::ld(T, l * wp + c);
-    P::fma(ar, e, tj[c]);
-    typename P::Acc pc;
-    P::init(pc);
-    P::fma(pc, e, ti[l]);
-    const typename P::V sc = warp_sum<P>(P::get(pc));
-    if (l == c) col = sc;
+  if (w <= 3) {
+    for (int c = 0; c < w; ++c) {
+      const typename P::V e = TileElem<P>::ld(T, l * wp + c);
+      P::fma(ar[0], e, tj[c]);
+      typename P::Acc pc;
+      P::init(pc);
+      P::fma(pc, e, ti[l]);
+      const typename P::V sc = warp_sum<P>(P::get(pc));
+      if (l == c) col = sc;
+    }
+    row = P::get(ar[0]);
+    return;
   }
-  row = P::get(ar);
+  int c = l % w;
+  for (int q = 0; q < w; ++q) {
+    P::fma(ar[0], TileElem<P>::ld(T, l * wp + c), tj[c]);
+    if (++c == w) c = 0;
+    if (++q == w) break;
+    P::fma(ar[1], TileElem<P>::ld(T, l * wp + c), tj[c]);
+    if (++c == w) c = 0;
+  }
+  row = P::add(P::get(ar[0]), P::get(ar[1]));
+  if (l < w) {
+    typename P::Acc ac[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) P::init(ac[u]);
+#pragma unroll
+    for (int r = 0; r < 32; ++r) P::fma(ac[r & 3], TileElem<P>::ld(T, r * wp + l), ti[r]);
+    col = P::add(P::add(P::get(ac[0]), P::get(ac[1])), P::add(P::get(ac[2]), P::get(ac[3])));
+  }
 }
 
 // Batched symmetric GEMV over the packed panels of SymTiles (one CTA per matrix): each warp
