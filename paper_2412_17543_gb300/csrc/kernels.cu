@@ -23,7 +23,7 @@
 
 namespace dd {
 
-// t_I = f_I - ck * (K [0; x_G])_I   (SCHUR: t = (K x)_I; CONDENSE: t = f_I; RECOVER: t = f_I - (K x)_I)
+// t_I = f_I - (K [0; x_G])_I   (CONDENSE: t = f_I)
 template <class P, int S>
 __global__ void __launch_bounds__(256) k_elem_interior(DevMesh m, int mode, const double* __restrict__ xg,
                                                        const double* __restrict__ f, double* __restrict__ tI) {
@@ -35,10 +35,10 @@ __global__ void __launch_bounds__(256) k_elem_interior(DevMesh m, int mode, cons
   const int16_t* code = m.lidx + (size_t)s * m.NL;
   const int* to = m.type_off + 6 * m.sub_type[s];
   const int64_t io = m.ioff[s];
-  // every interior output first gets its base value (0 or f_I)
+  // every interior output first gets its base value f_I
   for (int l = threadIdx.x; l < m.NL; l += blockDim.x) {
     int cd = code[l];
-    if (cd >= 0) tI[io + cd] = (mode == ELEM_SCHUR) ? 0.0 : f[free_index(m, s, l)];
+    if (cd >= 0) tI[io + cd] = f[free_index(m, s, l)];
   }
   if (mode == ELEM_CONDENSE) return;
   for (int l = threadIdx.x; l < m.NL; l += blockDim.x) {
@@ -52,17 +52,13 @@ __global__ void __launch_bounds__(256) k_elem_interior(DevMesh m, int mode, cons
     const int l = it[0];
     const double v = P::to_d(apply_item<P, S>(m, it, xl, kd));
     const int cd = code[l];
-    if (mode == ELEM_SCHUR)
-      tI[io + cd] = v;
-    else
-      tI[io + cd] = f[free_index(m, s, l)] - v;
+    tI[io + cd] = f[free_index(m, s, l)] - v;
   }
 }
 
-// y_G = (K [-s_I; x_G])_G  (SCHUR: x_G given; CONDENSE: x_G = 0)
+// y_G = -(K [s_I; 0])_G  (condensation)
 template <class P, int S>
-__global__ void __launch_bounds__(256) k_elem_interface(DevMesh m, int mode, const double* __restrict__ xg,
-                                                        const double* __restrict__ sI, double* __restrict__ yloc) {
+__global__ void __launch_bounds__(256) k_elem_interface(DevMesh m, const double* __restrict__ sI, double* __restrict__ yloc) {
   using V = typename P::V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* xl = reinterpret_cast<V*>(smem_raw);
@@ -74,7 +70,6 @@ __global__ void __launch_bounds__(256) k_elem_interface(DevMesh m, int mode, con
     int cd = code[l];
     V v = P::zero();
     if (cd >= 0) v = P::from_d(-sI[m.ioff[s] + cd]);
-    else if (cd != INT16_MIN && mode == ELEM_SCHUR) v = P::from_d(xg[m.gmap[m.goff[s] + (-1 - cd)]]);
     xl[l] = v;
   }
   build_kd_list<P, S>(m, s, m.type_bl + to[4], to[5] - to[4], kd);
@@ -97,14 +92,14 @@ static void elem_interior_dispatch(const DevMesh& m, int mode, const double* xg,
     k_elem_interior<P, 0><<<m.S, 256, smem, s>>>(m, mode, xg, f, tI);
 }
 template <class P>
-static void elem_interface_dispatch(const DevMesh& m, int mode, const double* xg, const double* sI, double* yloc,
+static void elem_interface_dispatch(const DevMesh& m, const double* sI, double* yloc,
                                     size_t smem, cudaStream_t s) {
   if (m.sx == 8 && m.sy == 8 && m.sz == 8)
-    k_elem_interface<P, 8><<<m.S, 256, smem, s>>>(m, mode, xg, sI, yloc);
+    k_elem_interface<P, 8><<<m.S, 256, smem, s>>>(m, sI, yloc);
   else if (m.sx == 4 && m.sy == 4 && m.sz == 4)
-    k_elem_interface<P, 4><<<m.S, 256, smem, s>>>(m, mode, xg, sI, yloc);
+    k_elem_interface<P, 4><<<m.S, 256, smem, s>>>(m, sI, yloc);
   else
-    k_elem_interface<P, 0><<<m.S, 256, smem, s>>>(m, mode, xg, sI, yloc);
+    k_elem_interface<P, 0><<<m.S, 256, smem, s>>>(m, sI, yloc);
 }
 
 void launch_elem_interior(const DevMesh& m, int mode, const double* xg, const double* f, double* tI,
@@ -118,14 +113,13 @@ void launch_elem_interior(const DevMesh& m, int mode, const double* xg, const do
   DD_CHECK_LAUNCH();
 }
 
-void launch_elem_interface(const DevMesh& m, int mode, const double* xg, const double* sI, double* yloc,
-                           cudaStream_t s) {
+void launch_elem_interface(const DevMesh& m, const double* sI, double* yloc, cudaStream_t s) {
   int NE = m.sx * m.sy * m.sz;
   size_t smem = (size_t)(m.NL + NE * 8) * 8;
   if (m.schur_prec == DD_PREC_DF64)
-    elem_interface_dispatch<PolDF>(m, mode, xg, sI, yloc, smem, s);
+    elem_interface_dispatch<PolDF>(m, sI, yloc, smem, s);
   else
-    elem_interface_dispatch<PolF64>(m, mode, xg, sI, yloc, smem, s);
+    elem_interface_dispatch<PolF64>(m, sI, yloc, smem, s);
   DD_CHECK_LAUNCH();
 }
 

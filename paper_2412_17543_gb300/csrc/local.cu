@@ -31,7 +31,7 @@ namespace dd {
 // ---------------------------------------------------------------------------
 // setup
 // ---------------------------------------------------------------------------
-LocalRowsHost build_local_rows(const Mesh1& M, const Level& L) {
+LocalRowsHost build_local_rows(const Mesh1& M, const Level& L, bool boundary_only) {
   LocalRowsHost R;
   const int S = M.S, NLx = M.NLx, NLy = M.NLy, NLz = M.NLz;
   struct Entry {
@@ -53,7 +53,25 @@ LocalRowsHost build_local_rows(const Mesh1& M, const Level& L) {
     types.emplace(pat, t);
     R.type[s] = t;
     const int nG = (int)(L.goff[s + 1] - L.goff[s]);
-    auto compact = [&](int l) { return code[l] >= 0 ? nG + code[l] : -1 - code[l]; };
+    // interior unknowns next to the interface, and their rank among these
+    std::vector<int> rank(M.NL, -1);
+    R.bnd.emplace_back();
+    for (int l = 0; l < M.NL; ++l) {
+      if (pat[l] != 1) continue;
+      const int a = l % NLx, b = (l / NLx) % NLy, c = l / (NLx * NLy);
+      bool next = false;
+      for (int z = std::max(c - 1, 0); z <= std::min(c + 1, NLz - 1); ++z)
+        for (int y = std::max(b - 1, 0); y <= std::min(b + 1, NLy - 1); ++y)
+          for (int x = std::max(a - 1, 0); x <= std::min(a + 1, NLx - 1); ++x)
+            next = next || pat[x + NLx * (y + NLy * z)] == 2;
+      if (!next) continue;
+      rank[l] = (int)R.bnd[t].size();
+      R.bnd[t].push_back(code[l]);
+    }
+    auto compact = [&](int l) {
+      if (code[l] < 0) return -1 - code[l];
+      return nG + (boundary_only ? rank[l] : code[l]);
+    };
     ell.emplace_back();
     const int nb_base = (int)R.nb.size();
     int range[4];
@@ -395,6 +413,51 @@ void launch_local_apply(const DevMesh& m, int mode, const double* xg, const doub
   else
     df ? local_go<PolDF, ELEM_RECOVER>(m, xg, f, out, s) : local_go<PolF64, ELEM_RECOVER>(m, xg, f, out, s);
   DD_CHECK_LAUNCH();
+}
+
+// ---------------------------------------------------------------------------
+// dense local solver: the same rows around a product with the boundary block of K_II^{-1}
+// ---------------------------------------------------------------------------
+// INTERIOR: t_B = K_BG x_G; else y = K_GG x_G - K_GB s_B
+template <class P, bool INTERIOR>
+__global__ void __launch_bounds__(LBS) k_rows(DevMesh m, const double* __restrict__ xg, const double* __restrict__ sB,
+                                              double* __restrict__ out) {
+  using V = typename P::V;
+  const LocalRows& R = m.rows;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* v = reinterpret_cast<V*>(smem_raw);  // [nG + nB]
+  const int s = blockIdx.x;
+  const int64_t go = m.goff[s], bo = R.boff[s];
+  const int nG = (int)(m.goff[s + 1] - go), nB = (int)(R.boff[s + 1] - bo);
+  const int* tr = R.trange + 5 * R.type[s];
+  const V* coef = static_cast<const V*>(R.coef) + R.coff[s];
+  for (int j = threadIdx.x; j < nG; j += LBS) v[j] = P::from_d(xg[m.gmap[go + j]]);
+  if (!INTERIOR)
+    for (int j = threadIdx.x; j < nB; j += LBS) v[nG + j] = P::from_d(-sB[bo + j]);
+  __syncthreads();
+  if (INTERIOR)
+    apply_rows<P>(R, tr[0], tr[1], tr[4], coef, v, [&](int o, V y) { out[bo + o - nG] = P::to_d(y); });
+  else
+    apply_rows<P>(R, tr[2], tr[3], tr[4], coef, v, [&](int o, V y) { out[go + o] = P::to_d(y); });
+}
+
+template <class P>
+static void schur_dense_go(const DevMesh& m, const double* xg, double* tB, double* sB, double* yloc, int* err,
+                           cudaStream_t s) {
+  const size_t smem = sizeof(typename P::V) * (size_t)m.rows.max_loc;
+  k_rows<P, true><<<m.S, LBS, smem, s>>>(m, xg, nullptr, tB);
+  DD_CHECK_LAUNCH();
+  launch_symv(m.KBB, m.rows.boff, tB, sB, err, s);
+  k_rows<P, false><<<m.S, LBS, smem, s>>>(m, xg, sB, yloc);
+  DD_CHECK_LAUNCH();
+}
+
+void launch_schur_dense(const DevMesh& m, const double* xg, double* tB, double* sB, double* yloc, int* err,
+                        cudaStream_t s) {
+  if (m.schur_prec == DD_PREC_DF64)
+    schur_dense_go<PolDF>(m, xg, tB, sB, yloc, err, s);
+  else
+    schur_dense_go<PolF64>(m, xg, tB, sB, yloc, err, s);
 }
 
 // ---------------------------------------------------------------------------

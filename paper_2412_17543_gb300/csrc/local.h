@@ -25,8 +25,15 @@ struct LocalRowsHost {
   std::vector<int16_t> nb;      // column position per entry, [slice][entry][32]
   std::vector<int64_t> coff;    // [S + 1] first coefficient of each subdomain
   std::vector<double> coef;     // per entry, FP64 sums over the bricks that hold both nodes
+  std::vector<std::vector<int>> bnd;  // per type: interior unknowns next to the interface (rows of pass 1)
 };
-LocalRowsHost build_local_rows(const Mesh1& M, const Level& L);
+// boundary_only: the interior part of the compact vector holds the unknowns of bnd only (dense
+// local solver), else all interior unknowns
+LocalRowsHost build_local_rows(const Mesh1& M, const Level& L, bool boundary_only);
+
+// Schur application of the dense local solver: y_loc from xg through t_B, s_B (scratch, rows.boff)
+void launch_schur_dense(const DevMesh& m, const double* xg, double* tB, double* sB, double* yloc, int* err,
+                        cudaStream_t s);
 
 // mode ELEM_SCHUR: out = y_loc from xg; ELEM_CONDENSE: out = y_loc from f (free-node vector);
 // ELEM_RECOVER: out = free-node solution from xg and f

@@ -72,9 +72,7 @@ extern "C" dd_status dd_schur_apply_noalloc(dd_ctx* ctx, const double* x, double
     } else if (m.local_solver == DD_LOCAL_FDM) {
       dd::launch_local_apply(m, dd::ELEM_SCHUR, x, nullptr, yloc, s);
     } else {
-      dd::launch_elem_interior(m, dd::ELEM_SCHUR, x, nullptr, tI, s);
-      dd::launch_symv(m.KIIinv, m.ioff, tI, sI, dd::context_err(ctx), s);
-      dd::launch_elem_interface(m, dd::ELEM_SCHUR, x, sI, yloc, s);
+      dd::launch_schur_dense(m, x, tI, sI, yloc, dd::context_err(ctx), s);
     }
     dd::launch_gather(m.n_gamma, m.gptr, m.gidx, yloc, nullptr, nullptr, y, s);
     return DD_OK;

@@ -224,12 +224,7 @@ void schur_local(dd_ctx* c, const double* x, cudaStream_t s) {
     launch_local_apply(c->mesh, ELEM_SCHUR, x, nullptr, c->w.yloc, s);
     return;
   }
-  launch_elem_interior(c->mesh, ELEM_SCHUR, x, nullptr, c->w.tI, s);
-  {
-    ProfScope pk(c, DD_PROF_SYMV_KII, s);
-    launch_symv(c->mesh.KIIinv, c->mesh.ioff, c->w.tI, c->w.sI, c->w.err, s);
-  }
-  launch_elem_interface(c->mesh, ELEM_SCHUR, x, c->w.sI, c->w.yloc, s);
+  launch_schur_dense(c->mesh, x, c->w.tI, c->w.sI, c->w.yloc, c->w.err, s);
 }
 
 void schur_apply(dd_ctx* c, const double* x, double* y, cudaStream_t s) {
@@ -244,7 +239,7 @@ void condense(dd_ctx* c, const double* f, double* b, cudaStream_t s) {
   } else {
     launch_elem_interior(c->mesh, ELEM_CONDENSE, nullptr, f, c->w.tI, s);
     launch_symv(c->mesh.KIIinv, c->mesh.ioff, c->w.tI, c->w.sI, c->w.err, s);
-    launch_elem_interface(c->mesh, ELEM_CONDENSE, nullptr, c->w.sI, c->w.yloc, s);
+    launch_elem_interface(c->mesh, c->w.sI, c->w.yloc, s);
   }
   launch_gather(c->n_gamma, c->mesh.gptr, c->mesh.gidx, c->w.yloc, f, c->mesh.gamma_free, b, s);
 }
@@ -596,7 +591,9 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
   tune_sym(c->b1.N, c->b1.goff, w.rloc, w.uloc, c->info.tune_symv_ms);
   if (c->mesh.local_solver != DD_LOCAL_FDM) {
     split_sym(c->mesh.KIIinv);
-    tune_sym(c->mesh.KIIinv, c->mesh.ioff, w.tI, w.sI, c->info.tune_kii_ms);
+    split_sym(c->mesh.KBB);
+    tune_sym(c->mesh.KBB, c->mesh.rows.boff, w.tI, w.sI, c->info.tune_kii_ms);
+    c->mesh.KIIinv.slots = c->mesh.KBB.slots;
   }
   zero(w.uC, c->b1.n_coarse * sizeof(double));
   tune_rows(c->b1.PhiT, c->b1.goff, c->b1.gmap, c->r, c->b1.coff, w.gloc, 1.0, nullptr, c->b1.D);
@@ -699,7 +696,8 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
     DevMesh& dm = c->mesh;
     std::vector<double> elem_madds, elem_nbl;  // per subdomain type (for the profiling counts)
     std::vector<int> elem_type;
-    std::vector<double> rows_madds;  // per subdomain: stored row entries (FDM)
+    std::vector<double> rows_madds;  // per subdomain: stored row entries
+    std::vector<int> bnd_n;          // per subdomain: interior unknowns next to the interface (dense)
     dm.nx = M.nx; dm.ny = M.ny; dm.nz = M.nz; dm.sx = M.sx; dm.sy = M.sy; dm.sz = M.sz;
     dm.Sx = M.Sx; dm.Sy = M.Sy; dm.Sz = M.Sz; dm.S = M.S;
     dm.fx0 = M.fx0; dm.fx1 = M.fx1; dm.fy0 = M.fy0; dm.fy1 = M.fy1; dm.fz0 = M.fz0; dm.fz1 = M.fz1;
@@ -805,40 +803,6 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
         dm.fdm_V = A.upload(Vd, s);
         dm.fdm_Dinv = A.upload(Dd, s);
       }
-      const LocalRowsHost R = build_local_rows(M, H->l1);
-      LocalRows& lr = dm.rows;
-      lr.type = A.upload(R.type, s);
-      lr.trange = A.upload(R.trange, s);
-      lr.sl_off = A.upload(R.sl_off, s);
-      lr.sl_out = A.upload(R.sl_out, s);
-      lr.sl_cnt = A.upload(R.sl_cnt, s);
-      lr.nb = A.upload(R.nb, s);
-      lr.coff = A.upload(R.coff, s);
-      if (opt->schur_prec == DD_PREC_DF64) {
-        std::vector<df64> cf(R.coef.size());
-#pragma omp parallel for schedule(static)
-        for (int64_t t = 0; t < (int64_t)cf.size(); ++t) cf[t] = df64_from_double(R.coef[t]);
-        lr.coef = A.upload(cf, s);
-      } else {
-        lr.coef = A.upload(R.coef, s);
-      }
-      std::vector<int> ifree((size_t)dm.n_int);
-      const int64_t Nfx = M.fx1 - M.fx0, Nfy = M.fy1 - M.fy0;
-      for (int i = 0; i < M.S; ++i) {
-        const int16_t* code = M.lidx.data() + (size_t)i * M.NL;
-        const int I = i % M.Sx, J = (i / M.Sx) % M.Sy, K = i / (M.Sx * M.Sy);
-        for (int l = 0; l < M.NL; ++l)
-          if (code[l] >= 0) {
-            const int a = l % M.NLx, b = (l / M.NLx) % M.NLy, q = l / (M.NLx * M.NLy);
-            ifree[H->l1.ioff[i] + code[l]] = (int)((I * M.sx + a - M.fx0) +
-                                                   Nfx * ((J * M.sy + b - M.fy0) + Nfy * (int64_t)(K * M.sz + q - M.fz0)));
-          }
-        lr.max_loc = std::max(lr.max_loc, (int)(H->l1.ioff[i + 1] - H->l1.ioff[i] + H->l1.goff[i + 1] - H->l1.goff[i]));
-      }
-      lr.ifree = A.upload(ifree, s);
-      // multiply-adds and element data of the profile: the rows' entries
-      rows_madds.resize(M.S);
-      for (int i = 0; i < M.S; ++i) rows_madds[i] = (double)(R.coff[i + 1] - R.coff[i]);
       dm.KIIinv.count = 0;
     } else {
       std::vector<const double*> mats;
@@ -848,6 +812,68 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
         dims.push_back(H->l1.sub[i].nI);
       }
       dm.KIIinv = upload_sym(A, mats, dims, opt->schur_prec == DD_PREC_DF64 ? DD_PREC_DF64 : DD_PREC_FP64, s);
+    }
+    {
+            const LocalRowsHost R = build_local_rows(M, H->l1, H->local_solver != DD_LOCAL_FDM);
+            LocalRows& lr = dm.rows;
+            lr.type = A.upload(R.type, s);
+            lr.trange = A.upload(R.trange, s);
+            lr.sl_off = A.upload(R.sl_off, s);
+            lr.sl_out = A.upload(R.sl_out, s);
+            lr.sl_cnt = A.upload(R.sl_cnt, s);
+            lr.nb = A.upload(R.nb, s);
+            lr.coff = A.upload(R.coff, s);
+            if (opt->schur_prec == DD_PREC_DF64) {
+              std::vector<df64> cf(R.coef.size());
+#pragma omp parallel for schedule(static)
+              for (int64_t t = 0; t < (int64_t)cf.size(); ++t) cf[t] = df64_from_double(R.coef[t]);
+              lr.coef = A.upload(cf, s);
+            } else {
+              lr.coef = A.upload(R.coef, s);
+            }
+            if (H->local_solver == DD_LOCAL_FDM) {
+        std::vector<int> ifree((size_t)dm.n_int);
+              const int64_t Nfx = M.fx1 - M.fx0, Nfy = M.fy1 - M.fy0;
+              for (int i = 0; i < M.S; ++i) {
+                const int16_t* code = M.lidx.data() + (size_t)i * M.NL;
+                const int I = i % M.Sx, J = (i / M.Sx) % M.Sy, K = i / (M.Sx * M.Sy);
+                for (int l = 0; l < M.NL; ++l)
+                  if (code[l] >= 0) {
+                    const int a = l % M.NLx, b = (l / M.NLx) % M.NLy, q = l / (M.NLx * M.NLy);
+                    ifree[H->l1.ioff[i] + code[l]] = (int)((I * M.sx + a - M.fx0) +
+                                                           Nfx * ((J * M.sy + b - M.fy0) + Nfy * (int64_t)(K * M.sz + q - M.fz0)));
+                  }
+                  }
+              lr.ifree = A.upload(ifree, s);
+            }
+      std::vector<int64_t> boff((size_t)M.S + 1, 0);
+      for (int i = 0; i < M.S; ++i) {
+        const int nG = (int)(H->l1.goff[i + 1] - H->l1.goff[i]), nI = (int)(H->l1.ioff[i + 1] - H->l1.ioff[i]);
+        const int nB = (int)R.bnd[R.type[i]].size();
+        boff[i + 1] = boff[i] + nB;
+        lr.max_loc = std::max(lr.max_loc, nG + (H->local_solver == DD_LOCAL_FDM ? nI : nB));
+      }
+      if (H->local_solver != DD_LOCAL_FDM) {
+        lr.boff = A.upload(boff, s);
+        std::vector<std::vector<double>> blocks(M.S);
+        std::vector<const double*> mats(M.S);
+        std::vector<int> dims(M.S);
+#pragma omp parallel for schedule(static)
+        for (int i = 0; i < M.S; ++i) {
+          const std::vector<int>& B = R.bnd[R.type[i]];
+          const int nb = (int)B.size(), nI = H->l1.sub[i].nI;
+          blocks[i].resize((size_t)nb * nb);
+          for (int a = 0; a < nb; ++a)
+            for (int b = 0; b < nb; ++b) blocks[i][(size_t)a * nb + b] = H->l1.sub[i].KIIinv[(size_t)B[a] * nI + B[b]];
+          mats[i] = blocks[i].data();
+          dims[i] = nb;
+        }
+        dm.KBB = upload_sym(A, mats, dims, opt->schur_prec == DD_PREC_DF64 ? DD_PREC_DF64 : DD_PREC_FP64, s);
+        bnd_n = dims;
+      }
+      // multiply-adds and element data of the profile: the rows' entries
+            rows_madds.resize(M.S);
+            for (int i = 0; i < M.S; ++i) rows_madds[i] = (double)(R.coff[i + 1] - R.coff[i]);
     }
     // ---- level-1 BDDC ----
     upload_bddc(A, H->l1, opt->precond_prec, c->b1, s);
@@ -950,7 +976,8 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
           const FdmSub& F = H->fdm[i];
           kii += (F.n[0] * F.n[0] + F.n[1] * F.n[1] + F.n[2] * F.n[2]) * 8.0 + a * 8.0 + 2 * a * 8.0;
         } else {
-          kii += a * (a + 1) / 2 * 8.0 + 2 * a * 8.0;
+          const double b = bnd_n[i];
+          kii += b * (b + 1) / 2 * 8.0 + 2 * b * 8.0;
         }
         nn += g * (g + 1) / 2 * (pp == DD_PREC_FP32 ? 4.0 : 8.0) + 2 * g * 8.0;
         // ensemble: the same matrix once, the members' vectors in the preconditioner type
@@ -967,7 +994,7 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
       const double n_flat = (double)H->l1.goff[M.S], n_g = (double)c->n_gamma;
       for (int i = 0; i < M.S; ++i) {
         const int t = elem_type[i];
-        const bool rows = H->local_solver == DD_LOCAL_FDM && !schur_fused_available(dm);
+        const bool rows = !schur_fused_available(dm);
         sm += rows ? rows_madds[i] : elem_madds[t];
         sb += rows ? rows_madds[i] * 8.0 : elem_nbl[t] * 3 * 8.0 + M.NL * 2.0;
         const double a = H->l1.sub[i].nI;
@@ -976,8 +1003,9 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
           sm += 2.0 * a * (F.n[0] + F.n[1] + F.n[2]) + a;
           sb += 243 * 8.0 + a * 8.0;
         } else {
-          sm += a * a;
-          sb += a * (a + 1) / 2 * 8.0;
+          const double b = bnd_n[i];
+          sm += b * b;
+          sb += b * (b + 1) / 2 * 8.0;
         }
       }
       sb += n_g * 8.0 + n_flat * (8.0 + 4.0) + n_flat * (8.0 + 8.0 + 4.0) + n_g * (8.0 + 4.0);
