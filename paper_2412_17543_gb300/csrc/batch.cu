@@ -535,10 +535,11 @@ void launch_symm_b(const SymTiles& A, const int64_t* voff, const void* in, void*
 
 // ---------------------------------------------------------------------------
 // batched row-major products with BW members (lane = member)
-//   k_bmm:   out_m[i] = alpha sum_j A_m[i][j] x_m[j]  -- a warp takes 4 rows, the row
-//            entries are loaded by the lanes (coalesced) and broadcast by shuffles
-//   k_bmm_t: out_m[j] = alpha sum_i A_m[i][j] x_m[i]  -- a warp takes 8 columns, 4 rows
-//            of them per load (lane = row * 8 + column)
+//   k_bmm:   out_m[i] = alpha sum_j A_m[i][j] x_m[j]  -- a warp takes 4 rows, 32 columns at a time
+//   k_bmm_t: out_m[j] = alpha sum_i A_m[i][j] x_m[i]  -- a warp takes 8 columns, 32 rows at a time
+// The entries are loaded coalesced, staged in the warp's shared memory and read back as
+// broadcast quads: half a shared-memory access per multiply-add. Broadcasting each entry by a shuffle
+// took more than one, and shuffles issue like shared-memory accesses.
 // ---------------------------------------------------------------------------
 template <class T>
 __device__ __forceinline__ T ld_x(const T* in, const int* in_map, int64_t io, int j, int lane) {
@@ -546,8 +547,13 @@ __device__ __forceinline__ T ld_x(const T* in, const int* in_map, int64_t io, in
   return in[src * BW + lane];
 }
 
+template <class T>
+struct alignas(16) Quad {
+  T v[4];
+};
+
 // STAGE: the item's input rows are first copied to shared memory ([rows][BW]) so the
-// inner loop runs on shared-memory loads and register shuffles only
+// inner loop runs on shared-memory loads only
 template <class T, bool STAGE>
 __global__ void __launch_bounds__(256) k_bmm(const int64_t* __restrict__ row0, const int* __restrict__ cols,
                                              const int64_t* __restrict__ moff, const T* __restrict__ M,
@@ -566,19 +572,34 @@ __global__ void __launch_bounds__(256) k_bmm(const int64_t* __restrict__ row0, c
     for (int t = threadIdx.x; t < C * BW; t += blockDim.x) xs[t] = ld_x(in, in_map, io, t / BW, t % BW);
     __syncthreads();
   }
+  __shared__ __align__(16) T as[8][4][32];
   for (int i0 = (blockIdx.y * nw + warp) * 4; i0 < R; i0 += gridDim.y * nw * 4) {
     T acc[4] = {0, 0, 0, 0};
-    for (int j0 = 0; j0 < C; j0 += 32) {
-      const int j = j0 + lane;
-      T a[4];
+    T a[4];
+    auto load = [&](int j) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) a[k] = (i0 + k < R && j < C) ? A[(int64_t)(i0 + k) * C + j] : (T)0;
+    };
+    load(lane);
+    for (int j0 = 0; j0 < C; j0 += 32) {
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 4; ++k) as[warp][k][lane] = a[k];
+      __syncwarp();
+      load(j0 + 32 + lane);  // the next chunk's entries while this one is used
       const int jn = min(32, C - j0);
 #pragma unroll 4
-      for (int jj = 0; jj < jn; ++jj) {
-        const T x = STAGE ? xs[(j0 + jj) * BW + lane] : ld_x(in, in_map, io, j0 + jj, lane);
+      for (int jj = 0; jj < jn; jj += 4) {
+        T x[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] = fma(__shfl_sync(0xffffffffu, a[k], jj), x, acc[k]);
+        for (int u = 0; u < 4; ++u)
+          x[u] = jj + u < jn ? (STAGE ? xs[(j0 + jj + u) * BW + lane] : ld_x(in, in_map, io, j0 + jj + u, lane)) : (T)0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const Quad<T> q = *reinterpret_cast<const Quad<T>*>(&as[warp][k][jj]);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc[k] = fma(q.v[u], x[u], acc[k]);
+        }
       }
     }
 #pragma unroll
@@ -608,18 +629,32 @@ __global__ void __launch_bounds__(256) k_bmm_t(const int64_t* __restrict__ row0,
     for (int t = threadIdx.x; t < R * BW; t += blockDim.x) xs[t] = ld_x(in, in_map, io, t / BW, t % BW);
     __syncthreads();
   }
-  const int lr = lane >> 3, lc = lane & 7;
+  __shared__ __align__(16) T as[8][32][8];
   for (int j0 = (blockIdx.y * nw + warp) * 8; j0 < C; j0 += gridDim.y * nw * 8) {
     T acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int i0 = 0; i0 < R; i0 += 4) {
-      const int ia = i0 + lr, ja = j0 + lc;
-      const T a = (ia < R && ja < C) ? A[(int64_t)ia * C + ja] : (T)0;
+    const int lr = lane >> 3, lc = lane & 7;
+    for (int i0 = 0; i0 < R; i0 += 32) {
+      T a[8];
 #pragma unroll
-      for (int rr = 0; rr < 4; ++rr) {
-        const int i = i0 + rr;
-        const T x = i < R ? (STAGE ? xs[i * BW + lane] : ld_x(in, in_map, io, i, lane)) : (T)0;
+      for (int u = 0; u < 8; ++u) {
+        const int i = i0 + 4 * u + lr;
+        a[u] = (i < R && j0 + lc < C) ? A[(int64_t)i * C + j0 + lc] : (T)0;
+      }
+      __syncwarp();
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] = fma(__shfl_sync(0xffffffffu, a, rr * 8 + k), x, acc[k]);
+      for (int u = 0; u < 8; ++u) as[warp][4 * u + lr][lc] = a[u];
+      __syncwarp();
+      const int in_ = min(32, R - i0);
+#pragma unroll 4
+      for (int r = 0; r < in_; ++r) {
+        const T x = STAGE ? xs[(i0 + r) * BW + lane] : ld_x(in, in_map, io, i0 + r, lane);
+        const Quad<T> q0 = *reinterpret_cast<const Quad<T>*>(&as[warp][r][0]);
+        const Quad<T> q1 = *reinterpret_cast<const Quad<T>*>(&as[warp][r][4]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          acc[k] = fma(q0.v[k], x, acc[k]);
+          acc[4 + k] = fma(q1.v[k], x, acc[4 + k]);
+        }
       }
     }
 #pragma unroll
@@ -684,48 +719,13 @@ void launch_bmm_t(const BatchedRows& B, const int64_t* in_off, const int* in_map
   DD_CHECK_LAUNCH();
 }
 
-// dense n x n times BW members: warp per row, lanes load the row, shuffles broadcast it
-template <class T>
-__global__ void __launch_bounds__(256) k_dense_mm(int n, const T* __restrict__ A, const T* __restrict__ x,
-                                                  T* __restrict__ y) {
-  const int lane = threadIdx.x & 31;
-  for (int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < n; row += (gridDim.x * blockDim.x) >> 5) {
-    const T* a = A + (int64_t)row * n;
-    T acc0 = 0, acc1 = 0;
-    for (int j0 = 0; j0 < n; j0 += 32) {
-      const T av = (j0 + lane < n) ? a[j0 + lane] : (T)0;
-      const int jn = min(32, n - j0);
-      int jj = 0;
-      for (; jj + 1 < jn; jj += 2) {
-        acc0 = fma(__shfl_sync(0xffffffffu, av, jj), x[(int64_t)(j0 + jj) * BW + lane], acc0);
-        acc1 = fma(__shfl_sync(0xffffffffu, av, jj + 1), x[(int64_t)(j0 + jj + 1) * BW + lane], acc1);
-      }
-      if (jj < jn) acc0 = fma(__shfl_sync(0xffffffffu, av, jj), x[(int64_t)(j0 + jj) * BW + lane], acc0);
-    }
-    y[(int64_t)row * BW + lane] = acc0 + acc1;
-  }
-}
-void launch_dense_mm(int prec, int n, const void* A, const void* x, void* y, cudaStream_t s) {
-  if (n == 0) return;
-  const int blocks = std::max(1, std::min(152 * 8, (n * 32 + 255) / 256));
-  if (prec == DD_PREC_FP32)
-    k_dense_mm<float><<<blocks, 256, 0, s>>>(n, (const float*)A, (const float*)x, (float*)y);
-  else
-    k_dense_mm<double><<<blocks, 256, 0, s>>>(n, (const double*)A, (const double*)x, (double*)y);
-  DD_CHECK_LAUNCH();
-}
-
-// The explicit coarse operator times BW members. A block takes CM_ROWS rows, its eight warps
+// Dense n x n operators (coarse inverses, the explicit coarse operator) times BW members. A block takes CM_ROWS rows, its eight warps
 // an eighth of the columns each (32 columns at a time: the rows' entries staged in shared
 // memory and read back as broadcast quads, the members' vectors coalesced from L2), and the
 // warps' sums are added in warp order.
 constexpr int CM_ROWS = 8;
 template <class T>
-struct alignas(16) Quad {
-  T v[4];
-};
-template <class T>
-__global__ void __launch_bounds__(256) k_coarse_mm(int n, const T* __restrict__ M, const T* __restrict__ x,
+__global__ void __launch_bounds__(256) k_dense_mm(int n, const T* __restrict__ M, const T* __restrict__ x,
                                                    T* __restrict__ y) {
   __shared__ __align__(16) T as[8][CM_ROWS][32];
   __shared__ T red[8][CM_ROWS][BW];
@@ -766,13 +766,13 @@ __global__ void __launch_bounds__(256) k_coarse_mm(int n, const T* __restrict__ 
     y[(int64_t)(i0 + warp) * BW + lane] = s;
   }
 }
-void launch_coarse_mm(int prec, int n, const void* M, const void* x, void* y, cudaStream_t s) {
+void launch_dense_mm(int prec, int n, const void* M, const void* x, void* y, cudaStream_t s) {
   if (n == 0) return;
   const int blocks = (n + CM_ROWS - 1) / CM_ROWS;
   if (prec == DD_PREC_FP32)
-    k_coarse_mm<float><<<blocks, 256, 0, s>>>(n, (const float*)M, (const float*)x, (float*)y);
+    k_dense_mm<float><<<blocks, 256, 0, s>>>(n, (const float*)M, (const float*)x, (float*)y);
   else
-    k_coarse_mm<double><<<blocks, 256, 0, s>>>(n, (const double*)M, (const double*)x, (double*)y);
+    k_dense_mm<double><<<blocks, 256, 0, s>>>(n, (const double*)M, (const double*)x, (double*)y);
   DD_CHECK_LAUNCH();
 }
 

@@ -105,9 +105,8 @@ void launch_wgather_tb(int prec, int64_t n, const int* ptr, const int* idx, cons
 // z[g][.] = sum over copies k of D_k (u_k + v_k)   (level-1 combine into the df64 Krylov vector)
 void launch_wgather_b(int prec, int64_t n, const int* ptr, const int* idx, const float* Df, const double* D,
                       const void* uloc, const void* vloc, df64* z, cudaStream_t s);
+// y = A x for a dense row-major n x n matrix
 void launch_dense_mm(int prec, int n, const void* A, const void* x, void* y, cudaStream_t s);
-// y = M x for the explicit coarse operator of small coarse spaces (row-major n x n)
-void launch_coarse_mm(int prec, int n, const void* M, const void* x, void* y, cudaStream_t s);
 // x = columns j0 .. j0 + BW - 1 of the n x n identity; rows of M's columns j0 .. from u
 void launch_unit_cols(int prec, int n, int j0, void* x, cudaStream_t s);
 void launch_store_cols(int prec, int n, int j0, const void* u, void* M, cudaStream_t s);

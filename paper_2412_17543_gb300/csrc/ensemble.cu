@@ -327,7 +327,7 @@ void precond_b(dd_ctx* c, const df64* r, df64* z, cudaStream_t s) {
            if (c->levels == 2)
              launch_dense_mm(c->b1.prec, c->b1.n_coarse, c->KCinv, g, u, ss);
            else if (dense_coarse_b(c))
-             launch_coarse_mm(c->b1.prec, c->b1.n_coarse, c->KCd, g, u, ss);
+             launch_dense_mm(c->b1.prec, c->b1.n_coarse, c->KCd, g, u, ss);
            else
              level2_b(c, g, u, ss);
          },
