@@ -575,9 +575,26 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
     }
   };
   auto split_sym = [&](SymTiles& A) {
-    if (A.count == 0 || A.count >= 152) return;
+    if (A.count == 0) return;
     const int nb = (A.max_n + 31) / 32;
-    const int want = (2 * 152 + A.count - 1) / A.count;
+    int want = (2 * 152 + A.count - 1) / A.count;
+    if (A.count >= 152) {
+      // FP64 products are bound by the SM's FP64 pipe (two FMAs per clock), so the launch lasts as long
+      // as the SM with the most matrix parts: take the number of parts with the least work there,
+      // each further part costing the vector it stages and combines (about 4 % of a matrix).
+      // FP32 and df64 products are bound by memory: one part each.
+      want = 1;
+      if (A.prec == DD_PREC_FP64) {
+        double best = 0.0;
+        for (int q = 1; q <= 4; ++q) {
+          const double load = std::ceil((double)A.count * q / 152.0) / q + 0.04 * (q - 1) * A.count / 152.0;
+          if (q == 1 || load < best) {
+            best = load;
+            want = q;
+          }
+        }
+      }
+    }
     A.split = std::max(1, std::min({8, want, nb * (nb + 1) / 2 / SYMV_WARPS_HOST}));
     if (A.split > 1 && !A.spart) {
       const int maxpad = nb * 32;
