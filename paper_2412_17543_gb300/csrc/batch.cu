@@ -552,6 +552,31 @@ struct alignas(16) Quad {
   T v[4];
 };
 
+// the item's input rows (all members) into shared memory, 16 bytes per load and four loads in flight
+template <class T>
+__device__ __forceinline__ void stage_rows(T* xs, const T* in, const int* in_map, int64_t io, int rows) {
+  constexpr int VPR = BW * (int)sizeof(T) / 16;  // 16-byte pieces of a row
+  uint4* dst = reinterpret_cast<uint4*>(xs);
+  const uint4* src = reinterpret_cast<const uint4*>(in);
+  const int nv = rows * VPR;
+  for (int t0 = threadIdx.x; t0 < nv; t0 += 4 * blockDim.x) {
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = t0 + u * blockDim.x;
+      if (t < nv) {
+        const int j = t / VPR;
+        v[u] = src[(in_map ? (int64_t)in_map[io + j] : io + j) * VPR + t % VPR];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = t0 + u * blockDim.x;
+      if (t < nv) dst[t] = v[u];
+    }
+  }
+}
+
 // STAGE: the item's input rows are first copied to shared memory ([rows][BW]) so the
 // inner loop runs on shared-memory loads only
 template <class T, bool STAGE>
@@ -569,7 +594,7 @@ __global__ void __launch_bounds__(256) k_bmm(const int64_t* __restrict__ row0, c
   const T* A = M + moff[mi];
   if (blockIdx.y * nw * 4 >= R) return;
   if (STAGE) {
-    for (int t = threadIdx.x; t < C * BW; t += blockDim.x) xs[t] = ld_x(in, in_map, io, t / BW, t % BW);
+    stage_rows(xs, in, in_map, io, C);
     __syncthreads();
   }
   __shared__ __align__(16) T as[8][4][32];
@@ -626,7 +651,7 @@ __global__ void __launch_bounds__(256) k_bmm_t(const int64_t* __restrict__ row0,
   const T* A = M + moff[mi];
   if (blockIdx.y * nw * 8 >= C) return;
   if (STAGE) {
-    for (int t = threadIdx.x; t < R * BW; t += blockDim.x) xs[t] = ld_x(in, in_map, io, t / BW, t % BW);
+    stage_rows(xs, in, in_map, io, R);
     __syncthreads();
   }
   __shared__ __align__(16) T as[8][32][8];
@@ -737,21 +762,24 @@ __global__ void __launch_bounds__(256) k_dense_mm(int n, const T* __restrict__ M
   for (int r = 0; r < CM_ROWS; ++r) acc[r] = (T)0;
   for (int ch = warp * chunks / 8; ch < (warp + 1) * chunks / 8; ++ch) {
     const int j0 = ch * 32;
-    __syncwarp();
+    // the chunk's entries and the members' values, all in flight together
+    T a[CM_ROWS], xv[32];
 #pragma unroll
     for (int r = 0; r < CM_ROWS; ++r)
-      as[warp][r][lane] = (i0 + r < n && j0 + lane < n) ? M[(int64_t)(i0 + r) * n + j0 + lane] : (T)0;
+      a[r] = (i0 + r < n && j0 + lane < n) ? M[(int64_t)(i0 + r) * n + j0 + lane] : (T)0;
+#pragma unroll
+    for (int q = 0; q < 32; ++q) xv[q] = j0 + q < n ? x[(int64_t)(j0 + q) * BW + lane] : (T)0;
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < CM_ROWS; ++r) as[warp][r][lane] = a[r];
     __syncwarp();
 #pragma unroll
     for (int q = 0; q < 32; q += 4) {
-      T xv[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) xv[u] = j0 + q + u < n ? x[(int64_t)(j0 + q + u) * BW + lane] : (T)0;
 #pragma unroll
       for (int r = 0; r < CM_ROWS; ++r) {
-        const Quad<T> a = *reinterpret_cast<const Quad<T>*>(&as[warp][r][q]);
+        const Quad<T> w = *reinterpret_cast<const Quad<T>*>(&as[warp][r][q]);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[r] = fma(a.v[u], xv[u], acc[r]);
+        for (int u = 0; u < 4; ++u) acc[r] = fma(w.v[u], xv[q + u], acc[r]);
       }
     }
   }
@@ -1004,14 +1032,19 @@ __global__ void __launch_bounds__(BRB) k_baxpy2(int64_t n, const double* sc, df6
   bfinalize_last(partials, 1, fin);
 }
 
+// reduction blocks for n rows: eight rows per warp or the full grid, whichever is less. On small
+// meshes the two levels of the finalization over 38 groups cost more than the rows themselves
+// (17214 rows: 15 us a reduction); by n alone, so the sums' order does not change between runs.
+static int bred_blocks(int64_t n) { return (int)std::min<int64_t>(NBLKB, std::max<int64_t>(64, (n + 63) / 64)); }
+
 void bvec_dots_fin(int64_t n, const df64* a0, const df64* b0, const df64* a1, const df64* b1, double* partials,
                    double* sc, int op, int flexible, unsigned* ticket, cudaStream_t s, const int* its) {
-  k_bdots<<<NBLKB, BRB, 0, s>>>(n, a0, b0, a1, b1, partials, BFinArgs{sc, op, flexible, its, ticket});
+  k_bdots<<<bred_blocks(n), BRB, 0, s>>>(n, a0, b0, a1, b1, partials, BFinArgs{sc, op, flexible, its, ticket});
   DD_CHECK_LAUNCH();
 }
 void bvec_axpy2_fin(int64_t n, double* sc, df64* x, const df64* p, df64* r, const df64* q, double* partials,
                     unsigned* ticket, cudaStream_t s) {
-  k_baxpy2<<<NBLKB, BRB, 0, s>>>(n, sc, x, p, r, q, partials, BFinArgs{sc, BFIN_RR, 0, nullptr, ticket});
+  k_baxpy2<<<bred_blocks(n), BRB, 0, s>>>(n, sc, x, p, r, q, partials, BFinArgs{sc, BFIN_RR, 0, nullptr, ticket});
   DD_CHECK_LAUNCH();
 }
 
