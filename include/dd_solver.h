@@ -224,7 +224,9 @@ dd_status dd_recover(dd_ctx* ctx, const double* f, const double* xg, double* x, 
  *    scratch entry read by a call is written earlier in the same call, so nothing
  *    needs clearing, but calls whose executions overlap on the GPU (different
  *    streams, or different contexts on one device) race on it and must be ordered
- *    by the caller. x, y: [n_gamma] device. */
+ *    by the caller. Of the context the kernels read the operators and write only the
+ *    error word, so the call may overlap the context's other work on another stream.
+ *    x, y: [n_gamma] device. */
 #define DD_NOALLOC_SCRATCH_BYTES (8u << 20)
 dd_status dd_schur_apply_noalloc(dd_ctx* ctx, const double* x, double* y, void* stream);
 

@@ -72,7 +72,11 @@ extern "C" dd_status dd_schur_apply_noalloc(dd_ctx* ctx, const double* x, double
     } else if (m.local_solver == DD_LOCAL_FDM) {
       dd::launch_local_apply(m, dd::ELEM_SCHUR, x, nullptr, yloc, s);
     } else {
-      dd::launch_schur_dense(m, x, tI, sI, yloc, dd::context_err(ctx), s);
+      // one CTA per matrix: the parts of a split product meet in partial vectors and tickets of
+      // the context, which a solve on another stream may be using
+      dd::DevMesh md = m;
+      md.KBB.split = 1;
+      dd::launch_schur_dense(md, x, tI, sI, yloc, dd::context_err(ctx), s);
     }
     dd::launch_gather(m.n_gamma, m.gptr, m.gidx, yloc, nullptr, nullptr, y, s);
     return DD_OK;
