@@ -107,9 +107,9 @@ void launch_wgather_b(int prec, int64_t n, const int* ptr, const int* idx, const
                       const void* uloc, const void* vloc, df64* z, cudaStream_t s);
 // y = A x for a dense row-major n x n matrix
 void launch_dense_mm(int prec, int n, const void* A, const void* x, void* y, cudaStream_t s);
-// x = columns j0 .. j0 + BW - 1 of the n x n identity; rows of M's columns j0 .. from u
-void launch_unit_cols(int prec, int n, int j0, void* x, cudaStream_t s);
-void launch_store_cols(int prec, int n, int j0, const void* u, void* M, cudaStream_t s);
+// x = columns j0 .. j0 + BW - 1 of the n x n identity; M's columns j0 .. (in the type of prec) from u
+void launch_unit_cols(int n, int j0, double* x, cudaStream_t s);
+void launch_store_cols(int prec, int n, int j0, const double* u, void* M, cudaStream_t s);
 void launch_map_gather_b(int prec, int64_t n, const int* map, const void* in, void* out, cudaStream_t s);
 void launch_map_scatter_b(int prec, int64_t n, const int* map, const void* in, void* out, cudaStream_t s);
 

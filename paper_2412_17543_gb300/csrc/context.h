@@ -36,7 +36,7 @@ struct dd_ctx {
   DevLevel2 l2{};
   const void* KCinv = nullptr;
   void* KCd = nullptr;          // [n_coarse][n_coarse] the level-2 BDDC as a matrix (small coarse spaces, three levels)
-  void* gCt = nullptr;          // [n_coarse] coarse residual in the preconditioner's type (with KCd)
+  double* gCt = nullptr;        // [n_coarse] scratch of its product
   Work w{};
   dd::BatchWork* bw = nullptr;  // ensemble workspace (allocated by the first batched solve)
   // Krylov buffers
@@ -180,7 +180,9 @@ namespace dd {
 // operators and steps of one solve (solver.cu)
 void schur_apply(dd_ctx* c, const double* x, double* y, cudaStream_t s);
 void precond_apply(dd_ctx* c, const double* r, double* z, cudaStream_t s);
-void build_coarse_dense(dd_ctx* c, cudaStream_t s);
+// whether the level-2 BDDC is applied as an explicit matrix, and its formation from FP64 operators
+bool coarse_dense_fits(const dd_ctx* c);
+void build_coarse_dense(dd_ctx* c, const dd::DevLevel2& ops, cudaStream_t s);
 void recycle_update(dd_ctx* c, dd_recycle* st, int l, cudaStream_t s);
 void check_err(dd_ctx* c, cudaStream_t s);
 void set_last_error(const std::string& msg);

@@ -234,8 +234,8 @@ void launch_coef_grad(const DevMesh& m, const double* x, const double* lam, doub
 // part[b] (b < nblk) = block maxima of |k_e - c_e| / |k_e| (c_e = exp(coef_e) when log)
 void launch_coef_mismatch(const DevMesh& m, const double* coef, int log, double* part, int nblk, cudaStream_t s);
 void launch_scatter_recover(const DevMesh& m, const double* xg, const double* sI, double* x, cudaStream_t s);
-// the explicit coarse operator of small coarse spaces: y = M x, x_j = sum of the copies of the
-// local coarse vectors (x and the sums in the type of prec); xs: [n] scratch of that type
+// the explicit coarse operator of small coarse spaces: y = M x (M in the type of prec), x_j = sum of
+// the copies of the local coarse vectors; xs: [n] scratch of 8-byte values
 void launch_coarse_gemv(int n, int prec, const void* M, const int* cptr, const int* cidx, const double* gloc,
                         void* xs, double* y, cudaStream_t s);
 void launch_restrict(int64_t nflat, const int* gmap, const double* D, const double* r, double* rloc, cudaStream_t s);

@@ -334,13 +334,16 @@ void precond_b(dd_ctx* c, const df64* r, df64* z, cudaStream_t s) {
          s);
 }
 
-// The scratch that the level-2 operators find through the context while the explicit matrix is
-// built; the context's own workspace and tile pointers are put back whatever happens.
+// The level-2 operators and scratch that level2_b finds through the context while the explicit
+// matrix is built; the context's own are put back whatever happens.
 struct ScratchLevel2 {
   dd_ctx* c;
   BatchWork* bw;
   DevLevel2 l2;
-  ScratchLevel2(dd_ctx* c_, BatchWork* tmp) : c(c_), bw(c_->bw), l2(c_->l2) { c->bw = tmp; }
+  ScratchLevel2(dd_ctx* c_, BatchWork* tmp, const DevLevel2& ops) : c(c_), bw(c_->bw), l2(c_->l2) {
+    c->bw = tmp;
+    c->l2 = ops;
+  }
   ~ScratchLevel2() {
     c->bw = bw;
     c->l2 = l2;
@@ -434,32 +437,40 @@ dd_status pcg_solve_b(dd_ctx* c, dd_recycle* st, double rtol, bool record, int n
 
 }  // namespace
 
+bool coarse_dense_fits(const dd_ctx* c) {
+  const int n = c->b1.n_coarse;
+  if (c->levels != 3 || n == 0 || n > COARSE_DENSE_MAX) return false;
+  // the CUDA-core tile kernel holds a matrix's vectors of BW members in shared memory
+  const int npad = (std::max(c->l2.KIIinv.max_n, c->l2.b.N.max_n) + 31) / 32 * 32;
+  return (size_t)npad * BW * sizeof(double) <= 227 * 1024;
+}
+
 // The level-2 BDDC of a small coarse space as one matrix: its columns from the operators
 // themselves, BW unit vectors at a time. On the 64^3 mesh (2863 coarse dofs) the coarse branch of one
-// preconditioner application was fourteen dependent launches; it is two now.
-void build_coarse_dense(dd_ctx* c, cudaStream_t s) {
+// preconditioner application was fourteen dependent launches; it is two now. The columns are
+// formed in FP64 whatever the preconditioner's type and rounded to it once: formed by FP32 operators
+// and vectors, the matrix took a whole FP32 application (64^3 and smaller) from 0.8e-7 .. 2e-7 to
+// 1e-7 .. 7e-7 from the FP64 one.
+void build_coarse_dense(dd_ctx* c, const DevLevel2& ops, cudaStream_t s) {
   const int n = c->b1.n_coarse, prec = c->b1.prec;
-  if (c->levels != 3 || n == 0 || n > COARSE_DENSE_MAX) return;
-  const size_t eb = prec == DD_PREC_FP32 ? 4 : 8;
-  const int npad = (std::max(c->l2.KIIinv.max_n, c->l2.b.N.max_n) + 31) / 32 * 32;
-  if ((size_t)npad * BW * eb > 227 * 1024) return;  // the CUDA-core tile kernel holds a matrix's vectors
   BatchWork tmp;
-  alloc_level2(c, tmp);
-  void* x = typed_vec(tmp.arena, prec, n);
-  void* u = typed_vec(tmp.arena, prec, n);
-  void* M = eb == 4 ? (void*)c->arena.alloc<float>((size_t)n * n) : (void*)c->arena.alloc<double>((size_t)n * n);
+  void* M = prec == DD_PREC_FP32 ? (void*)c->arena.alloc<float>((size_t)n * n)
+                                 : (void*)c->arena.alloc<double>((size_t)n * n);
+  double* x = tmp.arena.alloc<double>((size_t)n * BW);
+  double* u = tmp.arena.alloc<double>((size_t)n * BW);
   {
-    ScratchLevel2 scope(c, &tmp);
+    ScratchLevel2 scope(c, &tmp, ops);
+    alloc_level2(c, tmp);
     ensure_tiles(tmp.arena, c->l2.KIIinv, s);
     ensure_tiles(tmp.arena, c->l2.b.N, s);
     for (int j0 = 0; j0 < n; j0 += BW) {
-      launch_unit_cols(prec, n, j0, x, s);
+      launch_unit_cols(n, j0, x, s);
       level2_b(c, x, u, s);
       launch_store_cols(prec, n, j0, u, M, s);
     }
     DD_CUDA(cudaStreamSynchronize(s));
   }
-  c->gCt = eb == 4 ? (void*)c->arena.alloc<float>(n) : (void*)c->arena.alloc<double>(n);
+  c->gCt = c->arena.alloc<double>(n);
   c->KCd = M;
 }
 

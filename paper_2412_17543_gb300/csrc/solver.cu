@@ -211,6 +211,29 @@ const void* upload_dense(DeviceArena& A, const std::vector<double>& M, int prec)
   return d;
 }
 
+// the level-2 operators in the type of prec
+void upload_level2(DeviceArena& A, const HostSetup& H, int prec, DevLevel2& L, cudaStream_t s) {
+  const int rp = prec == DD_PREC_FP32 ? DD_PREC_FP32 : DD_PREC_FP64;
+  upload_bddc(A, H.l2, prec, L.b, s);
+  L.n_int = H.l2.ioff[H.l2.S];
+  L.ioff = A.upload(H.l2.ioff, s);
+  L.imap = A.upload(H.imap2, s);
+  L.gam_c = A.upload(H.gam2_c, s);
+  L.gam_c64 = A.upload(std::vector<int64_t>(H.gam2_c.begin(), H.gam2_c.end()), s);
+  std::vector<const double*> Ks, Es;
+  std::vector<int> nI, nG;
+  for (int j = 0; j < H.l2.S; ++j) {
+    Ks.push_back(H.l2.sub[j].KIIinv.data());
+    Es.push_back(H.l2.sub[j].E.data());
+    nI.push_back(H.l2.sub[j].nI);
+    nG.push_back(H.l2.sub[j].nG);
+  }
+  L.KIIinv = upload_sym(A, Ks, nI, rp, s);
+  L.E = upload_rows(A, Es, nI, nG, rp, false, s);
+  L.n3 = H.l2.n_coarse;
+  L.KC3inv = upload_dense(A, H.KC3inv, prec);
+}
+
 // ---------------------------------------------------------------------------
 // operators
 // ---------------------------------------------------------------------------
@@ -913,24 +936,7 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
       c->KCinv = upload_dense(A, H->KCinv, pp);
     } else {
       DevLevel2& L = c->l2;
-      upload_bddc(A, H->l2, pp, L.b, s);
-      L.n_int = H->l2.ioff[H->l2.S];
-      L.ioff = A.upload(H->l2.ioff, s);
-      L.imap = A.upload(H->imap2, s);
-      L.gam_c = A.upload(H->gam2_c, s);
-      L.gam_c64 = A.upload(std::vector<int64_t>(H->gam2_c.begin(), H->gam2_c.end()), s);
-      std::vector<const double*> Ks, Es;
-      std::vector<int> nI, nG;
-      for (int j = 0; j < H->l2.S; ++j) {
-        Ks.push_back(H->l2.sub[j].KIIinv.data());
-        Es.push_back(H->l2.sub[j].E.data());
-        nI.push_back(H->l2.sub[j].nI);
-        nG.push_back(H->l2.sub[j].nG);
-      }
-      L.KIIinv = upload_sym(A, Ks, nI, pp == DD_PREC_FP32 ? DD_PREC_FP32 : DD_PREC_FP64, s);
-      L.E = upload_rows(A, Es, nI, nG, pp == DD_PREC_FP32 ? DD_PREC_FP32 : DD_PREC_FP64, false, s);
-      L.n3 = H->l2.n_coarse;
-      L.KC3inv = upload_dense(A, H->KC3inv, pp);
+      upload_level2(A, *H, pp, L, s);
       w.gI2 = A.alloc<double>(L.n_int);
       w.u0I2 = A.alloc<double>(L.n_int);
       w.uI2 = A.alloc<double>(L.n_int);
@@ -982,7 +988,15 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
       for (auto& e : c->ev_aux) DD_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     }
     DD_CUDA(cudaStreamSynchronize(s));
-    build_coarse_dense(c.get(), s);
+    if (coarse_dense_fits(c.get())) {
+      DeviceArena t;
+      DevLevel2 ops = c->l2;
+      if (pp == DD_PREC_FP32) {
+        ops = DevLevel2{};
+        upload_level2(t, *H, DD_PREC_FP64, ops, s);
+      }
+      build_coarse_dense(c.get(), ops, s);
+    }
     {
       // algorithmic bytes of one K_II^{-1} application: the operator data read once and the
       // vectors in and out (dense: packed triangles; FDM: 1D eigenbases and D^{-1})
