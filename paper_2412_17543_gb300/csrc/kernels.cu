@@ -313,7 +313,10 @@ __device__ __forceinline__ df64 warp_sum<PolDF>(df64 v) {
 // diagonal block of height h stored as its packed upper triangle (row r starts at
 // off(r) = r h - r (r - 1) / 2): lane l < h returns sum_c T(l, c) x_c. The lower part is
 // read by symmetry in a first sweep over r (lanes l > r read the contiguous entries
-// T(r, l), at off(r) + l - r), the upper part in a second sweep along the lane's own row.
+// T(r, l), at off(r) + l - r), the upper part in a second sweep along the lane's own row,
+// from its far end to the diagonal: that product, the largest, is not carried through the
+// roundings of the others (the 218 unknowns of K_II^{-1} next to the interface, df64: 8.7e-15 with the
+// diagonal first, 3.2e-15 with it last; all 343 unknowns 7.1e-15 with it first).
 template <class P, int H>
 __device__ __forceinline__ typename P::V packed_diag_sweep(const unsigned char* T, const typename P::V* tv, int l,
                                                            int h) {
@@ -330,8 +333,7 @@ __device__ __forceinline__ typename P::V packed_diag_sweep(const unsigned char* 
   }
   const int base = l * hh - l * (l - 1) / 2;
 #pragma unroll
-  for (int t = 0; t < (H ? H : 32); ++t) {
-    if (!H && t >= hh) break;
+  for (int t = (H ? H : 32) - 1; t >= 0; --t) {
     if (l + t < hh) P::fma(a1, TileElem<P>::ld(T, base + t), tv[l + t]);
   }
   return P::add(P::get(a0), P::get(a1));
