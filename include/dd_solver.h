@@ -145,7 +145,7 @@ typedef struct {
   int32_t symv_slots;       /* bulk copies in flight per warp of the level-1 N_i product (timed at setup) */
   int32_t schur_threads;    /* threads per block of the fused Schur kernel (timed at setup; 0: not used) */
   float tune_symv_ms[3];    /* setup timings of the N_i product with 2, 3, 4 copies in flight (0: not timed) */
-  float tune_kii_ms[3];     /* the same for a dense K_II^{-1} */
+  float tune_kii_ms[3];     /* the same for the dense local solver's product with K_II^{-1} (DD_PROF_SYMV_KII) */
   float tune_schur_ms[3];   /* setup timings of the fused Schur kernel with 256, 352, 416 threads */
 } dd_info_t;
 
@@ -277,10 +277,15 @@ dd_status dd_adjoint(dd_ctx* ctx, const double* grad_x, const double* x, double*
 dd_status dd_coef_mismatch(dd_ctx* ctx, const double* coef, int32_t coef_is_log, double* max_rel_diff, void* stream);
 
 /* ---- profiling (CUDA events on the launching stream) ---- */
-enum { DD_PROF_SYMV_KII = 0,   /* batched K_II^{-1} application of the Schur operator (Sect. 3.1) */
+enum { DD_PROF_SYMV_KII = 0,   /* batched product of the Schur operator with K_II^{-1} (Sect. 3.1) of the dense
+                                  local solver, of which it needs the rows and columns of the unknowns next to the
+                                  interface; fast diagonalization applies K_II^{-1} inside its one kernel and
+                                  records none */
        DD_PROF_SYMV_N = 1,     /* batched constrained-Neumann GEMV of BDDC (eq. 9) */
-       DD_PROF_SCHUR = 2,      /* whole Schur-complement applications */
-       DD_PROF_PRECOND = 3,    /* whole BDDC applications */
+       DD_PROF_SCHUR = 2,      /* whole Schur-complement applications; in the iterations of a single sequence with
+                                  p^T q and the histories of p and q, which the assembling launch forms */
+       DD_PROF_PRECOND = 3,    /* whole BDDC applications; in the iterations of a single sequence with a Dirichlet
+                                  face with r^T z, r^T z_old and the history of z likewise */
        DD_PROF_RECYCLE = 4,    /* recycling updates between solves (Sect. 4.2) */
        DD_PROF_ENS_SCHUR = 5,  /* ensemble Schur-complement applications (dd_solve_batch) */
        DD_PROF_ENS_PRECOND = 6,/* ensemble BDDC applications */
@@ -291,7 +296,8 @@ enum { DD_PROF_SYMV_KII = 0,   /* batched K_II^{-1} application of the Schur ope
 typedef struct {
   double ms;                /* summed device time of the timed launches/regions */
   int64_t launches;         /* number of timed launches/regions */
-  double alg_bytes;         /* algorithmic bytes of one launch (matrix entries once, vectors in and out) */
+  double alg_bytes;         /* algorithmic bytes of one launch (matrix entries once, vectors in and out), the
+                               mean over the timed launches where these differ (DD_PROF_SCHUR, DD_PROF_PRECOND) */
   double alg_flops;         /* algorithmic floating-point operations of one launch (multiply-add = 2),
                                counted for the arithmetic-bound Schur operator; 0 where not counted */
 } dd_kernel_prof;

@@ -69,12 +69,14 @@ struct dd_ctx {
   struct Pending {
     int cls;
     cudaEvent_t a, b;
+    double extra;
   };
   std::vector<Pending> pending;
   std::vector<cudaEvent_t> pool;
   double prof_ms[DD_PROF_COUNT] = {0};
   int64_t prof_n[DD_PROF_COUNT] = {0};
   double prof_bytes[DD_PROF_COUNT] = {0};
+  double prof_extra[DD_PROF_COUNT] = {0};  // further bytes of the timed regions, summed
   double prof_flops[DD_PROF_COUNT] = {0};
   cudaEvent_t get_event() {
     if (!pool.empty()) {
@@ -92,6 +94,7 @@ struct dd_ctx {
       if (cudaEventElapsedTime(&ms, p.a, p.b) == cudaSuccess) {
         prof_ms[p.cls] += ms;
         prof_n[p.cls] += 1;
+        prof_extra[p.cls] += p.extra;
       }
       pool.push_back(p.a);
       pool.push_back(p.b);
@@ -120,13 +123,15 @@ struct dd_ctx {
 };
 
 namespace dd {
-// times the launches issued on `s` during its lifetime when profiling is on
+// times the launches issued on `s` during its lifetime when profiling is on; extra: bytes that this
+// region moves beyond those of its class (prof_bytes)
 struct ProfScope {
   dd_ctx* c;
   int cls;
   cudaStream_t s;
+  double extra;
   cudaEvent_t a = nullptr, b = nullptr;
-  ProfScope(dd_ctx* c_, int cls_, cudaStream_t s_) : c(c_), cls(cls_), s(s_) {
+  ProfScope(dd_ctx* c_, int cls_, cudaStream_t s_, double extra_ = 0.0) : c(c_), cls(cls_), s(s_), extra(extra_) {
     if (c->prof_on && cls >= 0 && cls < DD_PROF_COUNT) {
       a = c->get_event();
       b = c->get_event();
@@ -136,7 +141,7 @@ struct ProfScope {
   ~ProfScope() {
     if (a) {
       cudaEventRecord(b, s);
-      c->pending.push_back({cls, a, b});
+      c->pending.push_back({cls, a, b, extra});
     }
   }
 };

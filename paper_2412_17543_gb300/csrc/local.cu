@@ -451,23 +451,21 @@ __global__ void __launch_bounds__(LBS) k_rows(DevMesh m, const double* __restric
     apply_rows<P>(R, tr[2], tr[3], tr[4], coef, v, [&](int o, V y) { out[go + o] = P::to_d(y); });
 }
 
-template <class P>
-static void schur_dense_go(const DevMesh& m, const double* xg, double* tB, double* sB, double* yloc, int* err,
-                           cudaStream_t s) {
-  const size_t smem = sizeof(typename P::V) * (size_t)m.rows.max_loc;
-  k_rows<P, true><<<m.S, LBS, smem, s>>>(m, xg, nullptr, tB);
-  DD_CHECK_LAUNCH();
-  launch_symv(m.KBB, m.rows.boff, tB, sB, err, s);
-  k_rows<P, false><<<m.S, LBS, smem, s>>>(m, xg, sB, yloc);
+template <bool INTERIOR>
+static void rows_go(const DevMesh& m, const double* xg, const double* sB, double* out, cudaStream_t s) {
+  const size_t smem = sizeof(double) * (size_t)m.rows.max_loc;  // df64 values have the same size
+  if (m.schur_prec == DD_PREC_DF64)
+    k_rows<PolDF, INTERIOR><<<m.S, LBS, smem, s>>>(m, xg, sB, out);
+  else
+    k_rows<PolF64, INTERIOR><<<m.S, LBS, smem, s>>>(m, xg, sB, out);
   DD_CHECK_LAUNCH();
 }
 
-void launch_schur_dense(const DevMesh& m, const double* xg, double* tB, double* sB, double* yloc, int* err,
-                        cudaStream_t s) {
-  if (m.schur_prec == DD_PREC_DF64)
-    schur_dense_go<PolDF>(m, xg, tB, sB, yloc, err, s);
-  else
-    schur_dense_go<PolF64>(m, xg, tB, sB, yloc, err, s);
+void launch_rows_interior(const DevMesh& m, const double* xg, double* tB, cudaStream_t s) {
+  rows_go<true>(m, xg, nullptr, tB, s);
+}
+void launch_rows_interface(const DevMesh& m, const double* xg, const double* sB, double* yloc, cudaStream_t s) {
+  rows_go<false>(m, xg, sB, yloc, s);
 }
 
 // ---------------------------------------------------------------------------

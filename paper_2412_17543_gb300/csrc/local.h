@@ -31,9 +31,10 @@ struct LocalRowsHost {
 // local solver), else all interior unknowns
 LocalRowsHost build_local_rows(const Mesh1& M, const Level& L, bool boundary_only);
 
-// Schur application of the dense local solver: y_loc from xg through t_B, s_B (scratch, rows.boff)
-void launch_schur_dense(const DevMesh& m, const double* xg, double* tB, double* sB, double* yloc, int* err,
-                        cudaStream_t s);
+// rows of the dense local solver around the product s_B = K_BB t_B (vectors over rows.boff):
+// t_B = K_BG x_G, then y_loc = K_GG x_G - K_GB s_B
+void launch_rows_interior(const DevMesh& m, const double* xg, double* tB, cudaStream_t s);
+void launch_rows_interface(const DevMesh& m, const double* xg, const double* sB, double* yloc, cudaStream_t s);
 
 // mode ELEM_SCHUR: out = y_loc from xg; ELEM_CONDENSE: out = y_loc from f (free-node vector);
 // ELEM_RECOVER: out = free-node solution from xg and f

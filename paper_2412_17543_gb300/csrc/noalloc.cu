@@ -74,9 +74,11 @@ extern "C" dd_status dd_schur_apply_noalloc(dd_ctx* ctx, const double* x, double
     } else {
       // one CTA per matrix: the parts of a split product meet in partial vectors and tickets of
       // the context, which a solve on another stream may be using
-      dd::DevMesh md = m;
-      md.KBB.split = 1;
-      dd::launch_schur_dense(md, x, tI, sI, yloc, dd::context_err(ctx), s);
+      dd::SymTiles K = m.KBB;
+      K.split = 1;
+      dd::launch_rows_interior(m, x, tI, s);
+      dd::launch_symv(K, m.rows.boff, tI, sI, dd::context_err(ctx), s);
+      dd::launch_rows_interface(m, x, sI, yloc, s);
     }
     dd::launch_gather(m.n_gamma, m.gptr, m.gidx, yloc, nullptr, nullptr, y, s);
     return DD_OK;

@@ -247,7 +247,12 @@ void schur_local(dd_ctx* c, const double* x, cudaStream_t s) {
     launch_local_apply(c->mesh, ELEM_SCHUR, x, nullptr, c->w.yloc, s);
     return;
   }
-  launch_schur_dense(c->mesh, x, c->w.tI, c->w.sI, c->w.yloc, c->w.err, s);
+  launch_rows_interior(c->mesh, x, c->w.tI, s);
+  {
+    ProfScope pk(c, DD_PROF_SYMV_KII, s);
+    launch_symv(c->mesh.KBB, c->mesh.rows.boff, c->w.tI, c->w.sI, c->w.err, s);
+  }
+  launch_rows_interface(c->mesh, x, c->w.sI, c->w.yloc, s);
 }
 
 void schur_apply(dd_ctx* c, const double* x, double* y, cudaStream_t s) {
@@ -998,15 +1003,12 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
       build_coarse_dense(c.get(), ops, s);
     }
     {
-      // algorithmic bytes of one K_II^{-1} application: the operator data read once and the
-      // vectors in and out (dense: packed triangles; FDM: 1D eigenbases and D^{-1})
+      // algorithmic bytes of one product with the boundary block of K_II^{-1} (dense local solver; the FDM
+      // solver applies K_II^{-1} inside its one kernel): packed triangles once, the vectors in and out
       double kii = 0, nn = 0, nne = 0;
       for (int i = 0; i < M.S; ++i) {
-        double a = H->l1.sub[i].nI, g = H->l1.sub[i].nG;
-        if (H->local_solver == DD_LOCAL_FDM) {
-          const FdmSub& F = H->fdm[i];
-          kii += (F.n[0] * F.n[0] + F.n[1] * F.n[1] + F.n[2] * F.n[2]) * 8.0 + a * 8.0 + 2 * a * 8.0;
-        } else {
+        const double g = H->l1.sub[i].nG;
+        if (H->local_solver != DD_LOCAL_FDM) {
           const double b = bnd_n[i];
           kii += b * (b + 1) / 2 * 8.0 + 2 * b * 8.0;
         }
@@ -1576,7 +1578,9 @@ dd_status pcg_solve(dd_ctx* c, dd_recycle* st, double rtol, bool record, dd_stat
       update_p();
     } else {
       {
-        ProfScope ps(c, DD_PROF_PRECOND, bs);
+        // the Krylov dots read r and z_old, the history takes z
+        const bool kept = rec && c->ctl_host->its <= st->hmax;
+        ProfScope ps(c, DD_PROF_PRECOND, bs, 8.0 * n * (1 + (flex ? 1 : 0) + (kept ? 1 : 0)));
         precond_local(c, c->r, bs);
         vec_wgather_rz(n, c->b1.gptr, c->b1.gidx, c->b1.D, c->w.uloc, c->w.vloc, c->r, c->z, flex, c->partials, c->sc,
                        &c->ctl->its, c->fticket, recz, bs);
@@ -1586,7 +1590,9 @@ dd_status pcg_solve(dd_ctx* c, dd_recycle* st, double rtol, bool record, dd_stat
       update_p();
     }
     {
-      ProfScope ps(c, DD_PROF_SCHUR, bs);
+      // p^T q reads p, the histories take p and q
+      const bool kept = rec && c->ctl_host->its < st->hmax;
+      ProfScope ps(c, DD_PROF_SCHUR, bs, 8.0 * n * (1 + (kept ? 2 : 0)));
       schur_local(c, c->p, bs);
       vec_gather_pq(n, c->mesh.gptr, c->mesh.gidx, c->w.yloc, c->p, c->q, c->partials, c->sc, c->fticket, recp, recq,
                     bs);
@@ -1705,10 +1711,11 @@ dd_status dd_profile(dd_ctx* c, int32_t enable, dd_kernel_prof* prof, int64_t* l
       for (int k = 0; k < DD_PROF_COUNT; ++k) {
         prof[k].ms = c->prof_ms[k];
         prof[k].launches = c->prof_n[k];
-        prof[k].alg_bytes = c->prof_bytes[k];
+        prof[k].alg_bytes = c->prof_bytes[k] + (c->prof_n[k] ? c->prof_extra[k] / (double)c->prof_n[k] : 0.0);
         prof[k].alg_flops = c->prof_flops[k];
         c->prof_ms[k] = 0;
         c->prof_n[k] = 0;
+        c->prof_extra[k] = 0;
       }
     }
     if (launches) *launches = g_launches.exchange(0);
