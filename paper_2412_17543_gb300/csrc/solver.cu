@@ -1529,9 +1529,11 @@ dd_status pcg_solve(dd_ctx* c, dd_recycle* st, double rtol, bool record, dd_stat
   const float* Wf = (k && st->wf_valid) ? st->Wf : nullptr;
   DD_CUDA(cudaMemsetAsync(c->sc, 0, SC_COUNT * sizeof(double), s));
   // deflation of one iteration streams A W (df64) and W (df64 or FP32) once each, and z, p
-  // (read) and p (written); the Krylov dots r^T z (and r^T z_old) run in the same window
+  // (read) and p (written); without a Dirichlet face the Krylov dots r^T z (and r^T z_old) run in
+  // the same window, else they are formed with z
   c->prof_bytes[DD_PROF_DEFL] =
-      ((double)k * (8.0 + (Wf ? 4.0 : 8.0)) + 3.0 * 8.0 + (o.flexible ? 4.0 : 2.0) * 8.0) * (double)n;
+      ((double)k * (8.0 + (Wf ? 4.0 : 8.0)) + 3.0 * 8.0 + (c->neumann ? (o.flexible ? 4.0 : 2.0) * 8.0 : 0.0)) *
+      (double)n;
   if (k) {
     // x_0 = x_{-1} + W (W^T A W)^{-1} W^T (b - A x_{-1})   (assures W^T r_0 = 0)
     schur_apply(c, c->xg, c->q, s);

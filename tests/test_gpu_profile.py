@@ -62,3 +62,20 @@ def test_bytes_of_the_iterations(flexible, k):
     extra = (prof["precond_apply"][2] - alone["precond_apply"][2]) * prof["precond_apply"][1]
     assert extra == pytest.approx(its * n * (1 + flexible + kept), rel=1e-9)
     S.close()
+
+
+def test_bytes_of_the_deflation():
+    """k columns of A W (df64) and of W (FP64 preconditioner: df64), z and p in, p out; the Krylov dots are formed
+    with z."""
+    m = make_mesh(16, 4, 1.08, 20.0)
+    S = P.Solver(m, levels=2, use_corners=1, use_edges=1, use_faces=1)
+    rec = S.recycler(4)
+    F = load_sequence(m, 3, 3)
+    for t in range(2):
+        S.solve(T(F[t]), rec, rtol=1e-8)
+    S.profile(True)
+    _, st = S.solve(T(F[2]), rec, rtol=1e-8)
+    prof, _ = S.profile(False)
+    assert st["recycled_k"] == 4 and prof["deflation"][1] == st["iters"]
+    assert prof["deflation"][2] == pytest.approx((4 * 16.0 + 24.0) * S.n_gamma, rel=1e-12)
+    S.close()
