@@ -49,7 +49,9 @@ struct BatchWork {
   LoopCtl* ctl = nullptr;             // device-resident loop control
   LoopCtl* ctl_host = nullptr;        // pinned mirror
   double* alphas = nullptr;           // [maxit] member 0's step lengths
-  int nact = BW;  // members of the current call; the local operators skip chunks of padded members
+  // members that the local operators of the current call form: the call's own, rounded up to whole
+  // chunks (fast diagonalization), else all. One captured loop per value
+  int nact = BW;
   // members per CTA of the FDM subdomain operators (chosen by timing at the first ensemble call on
   // 8^3 df64 subdomains), and the timings (ms); elem_rc: the element passes' members per pass, as
   // the option asks (the FDM operators have no separate element pass)

@@ -121,6 +121,12 @@ void select_shapes(dd_ctx* c, cudaStream_t s) {
   B.fdm_rc = B.fdm_ms[0] < B.fdm_ms[1] ? 4 : 8;
 }
 
+int member_slots(const dd_ctx* c, int nrhs) {
+  if (c->mesh.local_solver != DD_LOCAL_FDM) return BW;
+  const int rc = c->bw->fdm_rc;
+  return (nrhs + rc - 1) / rc * rc;
+}
+
 // whether the ensemble applies the level-2 BDDC as the explicit matrix
 bool dense_coarse_b(const dd_ctx* c) { return c->KCd && c->b1.n_coarse <= COARSE_DENSE_MAX_B; }
 
@@ -486,6 +492,8 @@ dd_status dd_recycle_create_batch(dd_ctx* c, int32_t k, int32_t strategy, double
   rc = guard_call([&] {
     dd_recycle* st = *out;
     st->nrhs = BW;
+    // calls of changing width: a loop per chunk count (member_slots), of at least four members each
+    st->loop.keep(BW / 4);
     st->xg_prev_b = st->arena.alloc<df64>((size_t)c->n_gamma * BW);
     DD_CUDA(cudaMemset(st->xg_prev_b, 0, (size_t)c->n_gamma * BW * sizeof(df64)));
   });
@@ -510,7 +518,7 @@ static dd_status batch_op(dd_ctx* c, int32_t nrhs, const double* X, double* Y, v
   return guard_call([&] {
     cudaStream_t s = (cudaStream_t)stream;
     BatchWork& B = batch_work(c, s);
-    B.nact = nrhs;
+    B.nact = member_slots(c, nrhs);
     launch_pack_in(c->n_gamma, nrhs, X, B.p, s);
     if (precond)
       precond_b(c, B.p, B.q, s);
@@ -548,7 +556,7 @@ dd_status dd_solve_batch(dd_ctx* c, int32_t nrhs, const double* F, double* X, do
     cudaStream_t s = (cudaStream_t)stream;
     BatchWork& B = batch_work(c, s);
     DD_CUDA(cudaEventRecord(c->ev0, s));
-    B.nact = nrhs;
+    B.nact = member_slots(c, nrhs);
     launch_pack_in(c->n_free, nrhs, F, B.F, s);
     condense_b(c, B.F, B.bvec, s);
     copy_b(B.xg, st->xg_prev_b, c->n_gamma, s);

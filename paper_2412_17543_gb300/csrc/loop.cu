@@ -126,75 +126,91 @@ void launch_record_col0(const LoopCtl* ctl, const df64* src, double* dst, int64_
 }
 
 LoopGraph::~LoopGraph() {
-  reset();
+  for (Captured& c : held_) destroy(c);
   if (cap_) cudaStreamDestroy(cap_);
 }
 
-void LoopGraph::reset() {
-  if (exec_) cudaGraphExecDestroy(exec_);
-  if (graph_) cudaGraphDestroy(graph_);
-  exec_ = nullptr;
-  graph_ = nullptr;
-  key_.clear();
+void LoopGraph::destroy(Captured& c) {
+  if (c.exec) cudaGraphExecDestroy(c.exec);
+  if (c.graph) cudaGraphDestroy(c.graph);
+  c = Captured{};
+}
+
+LoopGraph::Captured LoopGraph::capture(const std::vector<uint64_t>& key, const Body& body, LoopCtl* ctl) {
+  if (!cap_) DD_CUDA(cudaStreamCreateWithFlags(&cap_, cudaStreamNonBlocking));
+  Captured c;
+  c.key = key;
+  try {
+    DD_CUDA(cudaGraphCreate(&c.graph, 0));
+    cudaGraphConditionalHandle h;
+    DD_CUDA(cudaGraphConditionalHandleCreate(&h, c.graph, 0, 0));
+    // gate node: the condition starts from ctl->go, which the stream set before the launch
+    cudaGraphNode_t gate;
+    {
+      const LoopCtl* cctl = ctl;
+      void* args[] = {(void*)&cctl, (void*)&h};
+      cudaKernelNodeParams kp{};
+      kp.func = (void*)k_loop_gate;
+      kp.gridDim = dim3(1);
+      kp.blockDim = dim3(1);
+      kp.sharedMemBytes = 0;
+      kp.kernelParams = args;
+      kp.extra = nullptr;
+      DD_CUDA(cudaGraphAddKernelNode(&gate, c.graph, nullptr, 0, &kp));
+    }
+    cudaGraphNodeParams cp{};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = h;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    cudaGraphNode_t cond;
+    DD_CUDA(cudaGraphAddNode(&cond, c.graph, &gate, nullptr, 1, &cp));
+    cudaGraph_t bodyg = cp.conditional.phGraph_out[0];
+    DD_CUDA(cudaStreamBeginCaptureToGraph(cap_, bodyg, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+    const int64_t l0 = launch_counter();
+    try {
+      body(cap_, h, true);
+    } catch (...) {
+      cudaGraph_t g2 = nullptr;
+      cudaStreamEndCapture(cap_, &g2);
+      cudaGetLastError();
+      throw;
+    }
+    // captured launches are counted when the graph runs them
+    c.body_launches = launch_counter() - l0;
+    add_launches(-c.body_launches);
+    cudaGraph_t g2 = nullptr;
+    DD_CUDA(cudaStreamEndCapture(cap_, &g2));
+    // kernel nodes keep the priority of the stream they were captured from (the BDDC
+    // coarse branch runs ahead of the level-1 N_i blocks, as in the host-issued loop)
+    DD_CUDA(cudaGraphInstantiate(&c.exec, c.graph, cudaGraphInstantiateFlagUseNodePriority));
+  } catch (...) {
+    destroy(c);
+    throw;
+  }
+  ++captures_;
+  return c;
 }
 
 void LoopGraph::run(const std::vector<uint64_t>& key, const Body& body, LoopCtl* ctl, LoopCtl* ctl_host,
                     bool use_graph, cudaStream_t s, const std::function<void()>& after_pass) {
   if (use_graph) {
-    if (!exec_ || key != key_) {
-      reset();
-      if (!cap_) DD_CUDA(cudaStreamCreateWithFlags(&cap_, cudaStreamNonBlocking));
-      DD_CUDA(cudaGraphCreate(&graph_, 0));
-      cudaGraphConditionalHandle h;
-      DD_CUDA(cudaGraphConditionalHandleCreate(&h, graph_, 0, 0));
-      // gate node: the condition starts from ctl->go, which the stream set before the launch
-      cudaGraphNode_t gate;
-      {
-        const LoopCtl* cctl = ctl;
-        void* args[] = {(void*)&cctl, (void*)&h};
-        cudaKernelNodeParams kp{};
-        kp.func = (void*)k_loop_gate;
-        kp.gridDim = dim3(1);
-        kp.blockDim = dim3(1);
-        kp.sharedMemBytes = 0;
-        kp.kernelParams = args;
-        kp.extra = nullptr;
-        DD_CUDA(cudaGraphAddKernelNode(&gate, graph_, nullptr, 0, &kp));
+    auto it = std::find_if(held_.begin(), held_.end(), [&](const Captured& c) { return c.key == key; });
+    if (it == held_.end()) {
+      // room first: the graphs that the stream still runs were waited for by their calls
+      while (!held_.empty() && held_.size() >= keep_) {
+        destroy(held_.front());
+        held_.erase(held_.begin());
       }
-      cudaGraphNodeParams cp{};
-      cp.type = cudaGraphNodeTypeConditional;
-      cp.conditional.handle = h;
-      cp.conditional.type = cudaGraphCondTypeWhile;
-      cp.conditional.size = 1;
-      cudaGraphNode_t cond;
-      DD_CUDA(cudaGraphAddNode(&cond, graph_, &gate, nullptr, 1, &cp));
-      cudaGraph_t bodyg = cp.conditional.phGraph_out[0];
-      DD_CUDA(cudaStreamBeginCaptureToGraph(cap_, bodyg, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-      const int64_t l0 = launch_counter();
-      try {
-        body(cap_, h, true);
-      } catch (...) {
-        cudaGraph_t g2 = nullptr;
-        cudaStreamEndCapture(cap_, &g2);
-        cudaGetLastError();
-        reset();
-        throw;
-      }
-      // captured launches are counted when the graph runs them
-      body_launches_ = launch_counter() - l0;
-      add_launches(-body_launches_);
-      cudaGraph_t g2 = nullptr;
-      DD_CUDA(cudaStreamEndCapture(cap_, &g2));
-      // kernel nodes keep the priority of the stream they were captured from (the BDDC
-      // coarse branch runs ahead of the level-1 N_i blocks, as in the host-issued loop)
-      DD_CUDA(cudaGraphInstantiate(&exec_, graph_, cudaGraphInstantiateFlagUseNodePriority));
-      key_ = key;
-      ++captures_;
+      held_.push_back(capture(key, body, ctl));
+    } else {
+      std::rotate(it, it + 1, held_.end());
     }
-    DD_CUDA(cudaGraphLaunch(exec_, s));
+    const Captured& c = held_.back();
+    DD_CUDA(cudaGraphLaunch(c.exec, s));
     DD_CUDA(cudaMemcpyAsync(ctl_host, ctl, sizeof(LoopCtl), cudaMemcpyDeviceToHost, s));
     DD_CUDA(cudaStreamSynchronize(s));
-    add_launches(1 + (int64_t)ctl_host->its * body_launches_);  // gate + iterations
+    add_launches(1 + (int64_t)ctl_host->its * c.body_launches);  // gate + iterations
     return;
   }
   DD_CUDA(cudaMemcpyAsync(ctl_host, ctl, sizeof(LoopCtl), cudaMemcpyDeviceToHost, s));

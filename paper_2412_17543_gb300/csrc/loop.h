@@ -54,8 +54,9 @@ void launch_record(const RecDst& rec, const double* src, int64_t n, cudaStream_t
 void launch_record_col0(const LoopCtl* ctl, const df64* src, double* dst, int64_t n, int limit, int inclusive,
                         cudaStream_t s);
 
-// One captured loop: the graph is rebuilt when the key (everything the body bakes into
-// its launches: sizes, basis width, buffer addresses, flags) changes.
+// Captured loops by key (everything the body bakes into its launches: sizes, basis width, buffer
+// addresses, flags): the last `keep` of them, one unless asked for more; a capture and its instantiation
+// take about 0.1 ms.
 class LoopGraph {
  public:
   using Body = std::function<void(cudaStream_t, cudaGraphConditionalHandle, bool in_graph)>;
@@ -63,6 +64,7 @@ class LoopGraph {
   LoopGraph(const LoopGraph&) = delete;
   LoopGraph& operator=(const LoopGraph&) = delete;
   ~LoopGraph();
+  void keep(size_t n) { keep_ = n; }
   // runs body while ctl->go (set on the stream before the call); ctl_host: pinned mirror,
   // current on return
   void run(const std::vector<uint64_t>& key, const Body& body, LoopCtl* ctl, LoopCtl* ctl_host, bool use_graph,
@@ -70,13 +72,18 @@ class LoopGraph {
   int captures() const { return captures_; }
 
  private:
-  void reset();
-  std::vector<uint64_t> key_;
-  cudaGraph_t graph_ = nullptr;
-  cudaGraphExec_t exec_ = nullptr;
+  struct Captured {
+    std::vector<uint64_t> key;
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    int64_t body_launches = 0;  // kernel launches of one captured iteration
+  };
+  static void destroy(Captured& c);
+  Captured capture(const std::vector<uint64_t>& key, const Body& body, LoopCtl* ctl);
+  std::vector<Captured> held_;  // least recently used first
+  size_t keep_ = 1;
   cudaStream_t cap_ = nullptr;  // capture stream: the caller's stream may be the legacy default stream
   int captures_ = 0;
-  int64_t body_launches_ = 0;  // kernel launches of one captured iteration
 };
 
 }  // namespace dd
