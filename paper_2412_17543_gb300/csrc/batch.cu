@@ -747,31 +747,41 @@ void launch_bmm_t(const BatchedRows& B, const int64_t* in_off, const int* in_map
 // Dense n x n operators (coarse inverses, the explicit coarse operator) times BW members. A block
 // takes CM_ROWS rows, its eight warps an eighth of the columns each (32 columns at a time: the rows'
 // entries staged in shared memory and read back as broadcast quads, the members' vectors
-// coalesced from L2). FP32 products are summed in FP32 over four columns; these sums, and
+// coalesced from L2). FP32 products are summed in FP32 over eight columns; these sums, and
 // the warps' in warp order, are added in df64. With FP32 sums over all columns of a warp the
 // explicit coarse operator took a whole FP32 application on smooth vectors from 4e-7 to 1.2e-6 from the FP64 one
 // (1115 coarse dofs).
 constexpr int CM_ROWS = 8;
 template <class T>
-struct QuadSum;
+struct EightSum;
 template <>
-struct QuadSum<float> {
+struct EightSum<float> {
   using S = df64;
   __device__ static S zero() { return {0.f, 0.f}; }
-  // a += a short sum; the low part stays of the order of the rounding of the high one
-  __device__ static void put(S& a, float t4) {
-    const df64 t = df64_two_sum(a.hi, t4);
-    a.hi = t.hi;
-    a.lo += t.lo;
+  // a += w . x; the low part stays of the order of the rounding of the high one
+  __device__ static void add8(S& a, const Quad<float>& w0, const Quad<float>& w1, const float* x) {
+    float t = w0.v[0] * x[0];
+#pragma unroll
+    for (int u = 1; u < 4; ++u) t = fmaf(w0.v[u], x[u], t);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) t = fmaf(w1.v[u], x[4 + u], t);
+    const df64 r = df64_two_sum(a.hi, t);
+    a.hi = r.hi;
+    a.lo += r.lo;
   }
   __device__ static S add(S a, S b) { return df64_add(a, b); }
   __device__ static float get(S a) { return a.hi + a.lo; }
 };
 template <>
-struct QuadSum<double> {
+struct EightSum<double> {
   using S = double;
   __device__ static S zero() { return 0.0; }
-  __device__ static void put(S& a, double t4) { a += t4; }
+  __device__ static void add8(S& a, const Quad<double>& w0, const Quad<double>& w1, const double* x) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a = fma(w0.v[u], x[u], a);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a = fma(w1.v[u], x[4 + u], a);
+  }
   __device__ static S add(S a, S b) { return a + b; }
   __device__ static double get(S a) { return a; }
 };
@@ -779,7 +789,7 @@ struct QuadSum<double> {
 template <class T>
 __global__ void __launch_bounds__(256) k_dense_mm(int n, const T* __restrict__ M, const T* __restrict__ x,
                                                    T* __restrict__ y) {
-  using CS = QuadSum<T>;
+  using CS = EightSum<T>;
   __shared__ __align__(16) T as[8][CM_ROWS][32];
   __shared__ typename CS::S red[8][CM_ROWS][BW];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -802,15 +812,11 @@ __global__ void __launch_bounds__(256) k_dense_mm(int n, const T* __restrict__ M
     for (int r = 0; r < CM_ROWS; ++r) as[warp][r][lane] = a[r];
     __syncwarp();
 #pragma unroll
-    for (int q = 0; q < 32; q += 4) {
+    for (int q = 0; q < 32; q += 8) {
 #pragma unroll
-      for (int r = 0; r < CM_ROWS; ++r) {
-        const Quad<T> w = *reinterpret_cast<const Quad<T>*>(&as[warp][r][q]);
-        T t4 = w.v[0] * xv[q];
-#pragma unroll
-        for (int u = 1; u < 4; ++u) t4 = fma(w.v[u], xv[q + u], t4);
-        CS::put(tot[r], t4);
-      }
+      for (int r = 0; r < CM_ROWS; ++r)
+        CS::add8(tot[r], *reinterpret_cast<const Quad<T>*>(&as[warp][r][q]),
+                 *reinterpret_cast<const Quad<T>*>(&as[warp][r][q + 4]), xv + q);
     }
   }
 #pragma unroll
