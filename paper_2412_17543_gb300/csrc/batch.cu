@@ -455,7 +455,12 @@ void launch_map_scatter_b(int prec, int64_t n, const int* map, const void* in, v
 // T^T X_bi into out_bj for the tiles of its columns, so every output block has one
 // writer and the sums are deterministic. Tiles are read row by row (broadcast loads).
 // ---------------------------------------------------------------------------
-constexpr int SYMM_WARPS = 16;  // a level-2 matrix (about 13 block rows) alone on its SM: 4 warps left it idle
+// Warps per matrix: one per block row up to eight, else sixteen. A warp without a block row takes room from
+// other matrices (FP64, 512 matrices of 4 and 5 block rows: 1034 and 1462 us with sixteen warps, 600 and 884 with
+// one each); a matrix of 13 block rows needs them all (512 matrices: FP64 5825 us with four warps, 4913 with
+// sixteen; FP32 786 with sixteen, 853 with thirteen).
+constexpr int SYMM_WARPS = 16;
+static int symm_warps(int npad) { return npad > 256 ? SYMM_WARPS : std::max(4, npad / 32); }
 
 template <class T>
 __global__ void __launch_bounds__(SYMM_WARPS * 32) k_symm_b(SymTiles A, const int64_t* __restrict__ voff,
@@ -465,7 +470,7 @@ __global__ void __launch_bounds__(SYMM_WARPS * 32) k_symm_b(SymTiles A, const in
   const int mtx = blockIdx.x;
   const int n = A.n[mtx];
   const int nb = (n + 31) / 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const int64_t vo = voff[mtx];
   for (int t = threadIdx.x; t < nb * 32 * BW; t += blockDim.x) acc[t] = (T)0;
   __syncthreads();
@@ -473,8 +478,8 @@ __global__ void __launch_bounds__(SYMM_WARPS * 32) k_symm_b(SymTiles A, const in
   int t = 0;
   for (int bi = 0; bi < nb; ++bi) {
     for (int bj = bi; bj < nb; ++bj, ++t) {
-      const bool own_row = (bi % SYMM_WARPS) == warp;
-      const bool own_col = bj != bi && (bj % SYMM_WARPS) == warp;
+      const bool own_row = (bi % warps) == warp;
+      const bool own_col = bj != bi && (bj % warps) == warp;
       if (!own_row && !own_col) continue;
       const T* Tl = tiles + (size_t)t * 1024;
       if (own_row) {
@@ -521,12 +526,12 @@ void launch_symm_b(const SymTiles& A, const int64_t* voff, const void* in, void*
   if (A.prec == DD_PREC_FP32) {
     const size_t smem = (size_t)npad * BW * 4;
     max_smem(k_symm_b<float>, smem);
-    k_symm_b<float><<<A.count, SYMM_WARPS * 32, smem, s>>>(A, voff, (const float*)in, (float*)out);
+    k_symm_b<float><<<A.count, symm_warps(npad) * 32, smem, s>>>(A, voff, (const float*)in, (float*)out);
   } else if (A.prec == DD_PREC_FP64) {
     const size_t smem = (size_t)npad * BW * 8;
     DD_REQUIRE(smem <= 227 * 1024, "ensemble: local matrix too large for the batched tile kernel");
     max_smem(k_symm_b<double>, smem);
-    k_symm_b<double><<<A.count, SYMM_WARPS * 32, smem, s>>>(A, voff, (const double*)in, (double*)out);
+    k_symm_b<double><<<A.count, symm_warps(npad) * 32, smem, s>>>(A, voff, (const double*)in, (double*)out);
   } else {
     throw Error(DD_INVALID_ARG, "ensemble: df64 dense tiles are not supported by the batched path");
   }
