@@ -512,8 +512,7 @@ def ensemble_main(args, wl, torch, pkg, dist, world, rank, local, dev, mesh, see
                 "ens_nmm": {"kernel": {1: "simt", 2: "tcgen05 3xTF32", 3: "tcgen05 BF16x3"}.get(S.info["ens_nmm"],
                                                                                                 "none"),
                             "tuning_ms": S.info["ens_nmm_ms"]},
-                "ens_shapes": {"element_members_per_pass": S.info["ens_elem_rc"],
-                               "fdm_members_per_block": S.info["ens_fdm_rc"]},
+                "ens_shapes": {"schur_members_per_block": S.info["ens_fdm_rc"]},
                 "batching_speedup": value / single["value"],
                 "e2e": e2e, "roofline": roof, "cpu_baseline": cpu, "clocks": clocks,
                 "gpu_launches": launches, "kernels": per_kernel}

@@ -103,10 +103,12 @@ typedef struct {
                                kernels timed on the first ensemble call, the fastest kept), DD_ENS_SIMT
                                (CUDA-core tiles), DD_ENS_TC (tensor cores, 3xTF32), DD_ENS_BF16X3
                                (tensor cores, bf16 operands in three slices, six products) */
-  int32_t ens_elem_rc;      /* members per pass of the ensemble element kernels of a DF64 operator on
-                               8^3-element subdomains: 0 (timed on the first ensemble call), 4, 8 or 16;
-                               any other shape of subdomain uses 8 */
-  int32_t ens_fdm_rc;       /* members per block of its ensemble fast diagonalization: 0 (timed), 4 or 8 */
+  int32_t ens_elem_rc;      /* 0, 4, 8 or 16: selects nothing. The element rows of an ensemble are applied in one kernel
+                               with the fast diagonalization, by blocks of ens_fdm_rc members; kept for callers that
+                               set it */
+  int32_t ens_fdm_rc;       /* members per block of the ensemble Schur operator of a DF64 operator on 8^3-element
+                               subdomains with fast diagonalization: 0 (timed on the first ensemble call), 4 or 8;
+                               any other uses 8 */
   int32_t loop_graph;       /* 1 (default): the PCG iterations of a solve run on the device as one launch
                                of a CUDA graph (conditional WHILE node; the stopping test is a kernel);
                                0: the host issues each iteration and reads the stopping test back.
@@ -135,8 +137,9 @@ typedef struct {
   int32_t ens_nmm;          /* ensemble N_i kernel in use: DD_ENS_SIMT, DD_ENS_TC or DD_ENS_BF16X3 (0
                                before the first ensemble call) */
   float ens_nmm_ms[3];      /* its selection timings (SIMT, 3xTF32, BF16x3; 0 when not timed), ms */
-  int32_t ens_elem_rc;      /* members per pass of the ensemble element kernels (0 before the first call) */
-  int32_t ens_fdm_rc;       /* members per block of the ensemble fast diagonalization (0 before) */
+  int32_t ens_elem_rc;      /* the option's value for a DF64 operator on 8^3-element subdomains, else ens_fdm_rc
+                               (0 before the first call) */
+  int32_t ens_fdm_rc;       /* members per block of the ensemble Schur operator (0 before) */
   int32_t neumann;          /* 1: no Dirichlet face (pure Neumann, Sect. 2): K is semidefinite with the
                                constants as null space; dd_solve projects the load vector onto the
                                range of K (removes its mean), keeps the preconditioned residuals

@@ -53,9 +53,9 @@ struct BatchWork {
   // chunks (fast diagonalization), else all. One captured loop per value
   int nact = BW;
   // members per CTA of the FDM subdomain operators (chosen by timing at the first ensemble call on
-  // 8^3 df64 subdomains), and the timings (ms); elem_rc: the element passes' members per pass, as
-  // the option asks (the FDM operators have no separate element pass)
-  int elem_rc = 8, fdm_rc = 8;
+  // 8^3 df64 subdomains), and the timings (ms)
+  int fdm_rc = 8;
+  int elem_rc = 0;  // what dd_get_info reports for the option ens_elem_rc; 0: fdm_rc
   float fdm_ms[2] = {0.f, 0.f};
   // symmetric products of the ensemble (level-1 N_i; level-2 K_II^{-1} and N): tensor-core
   // operand copy, the kernel in use, and the selection timings (SIMT, 3xTF32, BF16x3)

@@ -108,7 +108,7 @@ void select_shapes(dd_ctx* c, cudaStream_t s) {
   BatchWork& B = *c->bw;
   const DevMesh& m = c->mesh;
   if (m.schur_prec != DD_PREC_DF64 || !(m.sx == 8 && m.sy == 8 && m.sz == 8)) return;
-  if (c->opt.ens_elem_rc) B.elem_rc = c->opt.ens_elem_rc;
+  B.elem_rc = c->opt.ens_elem_rc;
   if (m.local_solver != DD_LOCAL_FDM) return;
   if (c->opt.ens_fdm_rc) {
     B.fdm_rc = c->opt.ens_fdm_rc;

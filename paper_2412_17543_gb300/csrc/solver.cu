@@ -1126,7 +1126,7 @@ dd_status dd_get_info(const dd_ctx* c, dd_info_t* info) {
   if (c->bw) {
     info->ens_nmm = c->bw->op[BOP_N1].kind;
     for (int v = 0; v < 3; ++v) info->ens_nmm_ms[v] = c->bw->op[BOP_N1].ms[v];
-    info->ens_elem_rc = c->bw->elem_rc;
+    info->ens_elem_rc = c->bw->elem_rc ? c->bw->elem_rc : c->bw->fdm_rc;
     info->ens_fdm_rc = c->bw->fdm_rc;
   }
   return DD_OK;

@@ -43,3 +43,19 @@ def test_changing_widths_are_captured_once(local, prec):
     assert any("cudaGraphLaunch" in n for n in names)
     assert not any("Instantiate" in n or "BeginCapture" in n for n in names)
     S.close()
+
+
+@pytest.mark.parametrize("fdm_rc", [4, 8])
+def test_members_per_block(fdm_rc):
+    """Counts that do and do not fill a block against single applications (df64: 1e-11 of the largest entry), and the
+    reported shapes: what the kernel runs with."""
+    m = make_mesh(16, 8, 1.3, 20.0)
+    S = P.Solver(m, levels=2, use_corners=1, use_edges=1, use_faces=1, schur_prec="df64", local_solver="fdm",
+                 ens_fdm_rc=fdm_rc)
+    X = torch.as_tensor(np.random.default_rng(fdm_rc).standard_normal((32, S.n_gamma)), device="cuda:0")
+    Y = torch.stack([S.schur_apply(x) for x in X])
+    for w in (1, 3, 4, 5, 8, 9, 31, 32):
+        Z = S.schur_apply_batch(X[:w].contiguous())
+        assert ((Z - Y[:w]).abs().amax(dim=1) <= 1e-11 * Y[:w].abs().amax(dim=1)).all()
+    assert (S.info["ens_elem_rc"], S.info["ens_fdm_rc"]) == (fdm_rc, fdm_rc)
+    S.close()
