@@ -960,7 +960,7 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
     c->xg = A.alloc<double>(nG);
     c->r = A.alloc<double>(nG);
     c->z = A.alloc<double>(nG);
-    c->zold = A.alloc<double>(nG);
+    if (c->neumann) c->zold = A.alloc<double>(nG);  // else z_old is read where z is written
     c->p = A.alloc<double>(nG);
     c->q = A.alloc<double>(nG);
     c->bvec = A.alloc<double>(nG);
