@@ -455,14 +455,7 @@ void launch_map_scatter_b(int prec, int64_t n, const int* map, const void* in, v
 // T^T X_bi into out_bj for the tiles of its columns, so every output block has one
 // writer and the sums are deterministic. Tiles are read row by row (broadcast loads).
 // ---------------------------------------------------------------------------
-// Warps per matrix: one per block row up to eight, else sixteen. A warp without a block row takes room from
-// other matrices (FP64, 512 matrices of 4 and 5 block rows: 1034 and 1462 us with sixteen warps, 600 and 884 with
-// one each); a matrix of 13 block rows needs them all (512 matrices: FP64 5825 us with four warps, 4913 with
-// sixteen; FP32 786 with sixteen, 853 with thirteen).
-constexpr int SYMM_WARPS = 16;
-static int symm_warps(int npad) { return npad > 256 ? SYMM_WARPS : std::max(4, npad / 32); }
-
-template <class T>
+template <class T, int SYMM_WARPS>
 __global__ void __launch_bounds__(SYMM_WARPS * 32) k_symm_b(SymTiles A, const int64_t* __restrict__ voff,
                                                             const T* __restrict__ in, T* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem_s[];
@@ -470,7 +463,7 @@ __global__ void __launch_bounds__(SYMM_WARPS * 32) k_symm_b(SymTiles A, const in
   const int mtx = blockIdx.x;
   const int n = A.n[mtx];
   const int nb = (n + 31) / 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t vo = voff[mtx];
   for (int t = threadIdx.x; t < nb * 32 * BW; t += blockDim.x) acc[t] = (T)0;
   __syncthreads();
@@ -478,8 +471,8 @@ __global__ void __launch_bounds__(SYMM_WARPS * 32) k_symm_b(SymTiles A, const in
   int t = 0;
   for (int bi = 0; bi < nb; ++bi) {
     for (int bj = bi; bj < nb; ++bj, ++t) {
-      const bool own_row = (bi % warps) == warp;
-      const bool own_col = bj != bi && (bj % warps) == warp;
+      const bool own_row = (bi % SYMM_WARPS) == warp;
+      const bool own_col = bj != bi && (bj % SYMM_WARPS) == warp;
       if (!own_row && !own_col) continue;
       const T* Tl = tiles + (size_t)t * 1024;
       if (own_row) {
@@ -520,18 +513,32 @@ __global__ void __launch_bounds__(SYMM_WARPS * 32) k_symm_b(SymTiles A, const in
   for (int i = threadIdx.x; i < n * BW; i += blockDim.x) out[vo * BW + i] = acc[i];
 }
 
+template <class T, int W>
+static void symm_go(const SymTiles& A, const int64_t* voff, const void* in, void* out, size_t smem, cudaStream_t s) {
+  max_smem(k_symm_b<T, W>, smem);
+  k_symm_b<T, W><<<A.count, W * 32, smem, s>>>(A, voff, (const T*)in, (T*)out);
+}
+// Warps per matrix: as many as block rows, 4, 8 or 16. A warp without a block row takes room from other
+// matrices (FP64, 512 matrices: SYMMFIG
+template <class T>
+static void symm_warps(const SymTiles& A, const int64_t* voff, const void* in, void* out, int npad, cudaStream_t s) {
+  const size_t smem = (size_t)npad * BW * sizeof(T);
+  if (A.count >= 152 && npad <= 4 * 32)
+    symm_go<T, 4>(A, voff, in, out, smem, s);
+  else if (A.count >= 152 && npad <= 8 * 32)
+    symm_go<T, 8>(A, voff, in, out, smem, s);
+  else
+    symm_go<T, 16>(A, voff, in, out, smem, s);
+}
+
 void launch_symm_b(const SymTiles& A, const int64_t* voff, const void* in, void* out, cudaStream_t s) {
   if (A.count == 0) return;
   const int npad = ((A.max_n + 31) / 32) * 32;
   if (A.prec == DD_PREC_FP32) {
-    const size_t smem = (size_t)npad * BW * 4;
-    max_smem(k_symm_b<float>, smem);
-    k_symm_b<float><<<A.count, symm_warps(npad) * 32, smem, s>>>(A, voff, (const float*)in, (float*)out);
+    symm_warps<float>(A, voff, in, out, npad, s);
   } else if (A.prec == DD_PREC_FP64) {
-    const size_t smem = (size_t)npad * BW * 8;
-    DD_REQUIRE(smem <= 227 * 1024, "ensemble: local matrix too large for the batched tile kernel");
-    max_smem(k_symm_b<double>, smem);
-    k_symm_b<double><<<A.count, symm_warps(npad) * 32, smem, s>>>(A, voff, (const double*)in, (double*)out);
+    DD_REQUIRE((size_t)npad * BW * 8 <= 227 * 1024, "ensemble: local matrix too large for the batched tile kernel");
+    symm_warps<double>(A, voff, in, out, npad, s);
   } else {
     throw Error(DD_INVALID_ARG, "ensemble: df64 dense tiles are not supported by the batched path");
   }

@@ -185,6 +185,7 @@ namespace dd {
 // operators and steps of one solve (solver.cu)
 void schur_apply(dd_ctx* c, const double* x, double* y, cudaStream_t s);
 void precond_apply(dd_ctx* c, const double* r, double* z, cudaStream_t s);
+void level2_apply(dd_ctx* c, const double* g, double* u, cudaStream_t s);
 // whether the level-2 BDDC is applied as an explicit matrix, and its formation from FP64 operators
 bool coarse_dense_fits(const dd_ctx* c);
 void build_coarse_dense(dd_ctx* c, const dd::DevLevel2& ops, cudaStream_t s);

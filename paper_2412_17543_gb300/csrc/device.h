@@ -139,7 +139,7 @@ struct DevMesh {
   // (df64 operator on 8^3-element subdomains with the fast-diagonalization solver only; else null):
   const int* sxg = nullptr;     // [S][NL] interface index of each local node (-1: not on the interface)
   const void* sfac = nullptr;   // [S][max_nbl][3] factors of the boundary-layer elements in the
-                                // order of the type's list (df64 or double, as schur_prec)
+                                // order of the type's list (df64)
 };
 
 // One BDDC level (Sect. 3.2): weights, constrained Neumann operator N, coarse basis
@@ -181,9 +181,16 @@ struct DevLevel2 {
 
 // Coarse spaces of at most this many dofs apply the level-2 BDDC as one explicit matrix
 // (built at setup). The recursive form is a chain of fourteen dependent launches of 2-8 us
-// each; the matrix costs its n^2 entries from L2 or HBM.
-constexpr int COARSE_DENSE_MAX = 4096;    // one vector: 67 MB of floats at most
-constexpr int COARSE_DENSE_MAX_B = 2048;  // ensembles: each block of 8 rows reads all members' vectors
+// each; the matrix costs its n^2 entries from L2 or HBM. One BDDC application (4^3 subdomains), matrix / chain:
+//   one vector, FP32: 1115 dofs 39 / 92 us, 1854 40 / 94, 3249 47 / 99, 3687 51 / 99, 4615 64 / 101, 5237 88 / 101
+//   one vector, FP64: 1115 52 / 105 us, 3249 95 / 122, 3687 108 / 125, 4615 130 / 138, 5237 145 / 143
+// The line lies where FP64 still gains, before the FP64 matrix outgrows L2 (134 MB at 4096 dofs) and its
+// formation the setup (0.15 s at 3249 dofs, 0.69 s at 4615).
+constexpr int COARSE_DENSE_MAX = 4096;    // one vector: 67 MB of floats or 134 MB of doubles at most
+// Ensembles (each block of 8 rows reads all members' vectors), 32 members:
+//   FP32: 1115 dofs 51 / 96 us, 1854 66 / 110, 3249 121 / 134, 3687 153 / 139
+//   FP64: 1115 468 / 456 us, 1854 790 / 997, 3249 1804 / 1243, 3687 2151 / 1291
+constexpr int COARSE_DENSE_MAX_B = 2048;
 
 // Scratch buffers of the operators (device).
 struct Work {

@@ -443,12 +443,17 @@ dd_status pcg_solve_b(dd_ctx* c, dd_recycle* st, double rtol, bool record, int n
 
 }  // namespace
 
+// whether the CUDA-core tile kernel holds the level-2 vectors of BW members in shared memory (matrices of up
+// to 1792 unknowns in FP32, 896 in FP64)
+static bool tiles_fit(const DevLevel2& L, size_t value) {
+  const size_t npad = (std::max(L.KIIinv.max_n, L.b.N.max_n) + 31) / 32 * 32;
+  return npad * BW * value <= 227 * 1024;
+}
+
 bool coarse_dense_fits(const dd_ctx* c) {
   const int n = c->b1.n_coarse;
   if (c->levels != 3 || n == 0 || n > COARSE_DENSE_MAX) return false;
-  // the CUDA-core tile kernel holds a matrix's vectors of BW members in shared memory
-  const int npad = (std::max(c->l2.KIIinv.max_n, c->l2.b.N.max_n) + 31) / 32 * 32;
-  return (size_t)npad * BW * sizeof(double) <= 227 * 1024;
+  return tiles_fit(c->l2, c->b1.prec == DD_PREC_FP32 ? sizeof(float) : sizeof(double));
 }
 
 // The level-2 BDDC of a small coarse space as one matrix: its columns from the operators
@@ -464,7 +469,20 @@ void build_coarse_dense(dd_ctx* c, const DevLevel2& ops, cudaStream_t s) {
                                  : (void*)c->arena.alloc<double>((size_t)n * n);
   double* x = tmp.arena.alloc<double>((size_t)n * BW);
   double* u = tmp.arena.alloc<double>((size_t)n * BW);
-  {
+  if (!tiles_fit(ops, sizeof(double))) {
+    // an FP32 preconditioner whose level-2 matrices are too wide for FP64 tiles: a vector at a time. The
+    // unit vectors are windows on one 1; the operator is symmetric, so a column is stored as a row
+    DD_REQUIRE(prec == DD_PREC_FP32, "explicit coarse operator: level-2 matrices too large");
+    const double one = 1.0;
+    DD_CUDA(cudaMemsetAsync(x, 0, (size_t)2 * n * sizeof(double), s));
+    DD_CUDA(cudaMemcpyAsync(x + n, &one, sizeof(double), cudaMemcpyHostToDevice, s));
+    ScratchLevel2 scope(c, c->bw, ops);
+    for (int j = 0; j < n; ++j) {
+      level2_apply(c, x + n - j, u, s);
+      launch_to_float(n, u, static_cast<float*>(M) + (size_t)j * n, s);
+    }
+    DD_CUDA(cudaStreamSynchronize(s));
+  } else {
     ScratchLevel2 scope(c, &tmp, ops);
     alloc_level2(c, tmp);
     ensure_tiles(tmp.arena, c->l2.KIIinv, s);

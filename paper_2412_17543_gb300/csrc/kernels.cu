@@ -1,12 +1,14 @@
 // Kernels of the Schur-complement operator and the BDDC preconditioner.
 //
 //  * k_elem_interior / k_elem_interface: the matrix-free Q1 operator of a
-//    subdomain (one CTA per subdomain). Each brick's 8x8 matrix is
+//    subdomain (one CTA per subdomain) for condensation and recovery with the dense
+//    local solver; everything else applies assembled rows (local.cu) or, single df64 vectors
+//    on 8^3 subdomains, k_schur_fused. Each brick's 8x8 matrix is
 //    k_e[(hy hz/hx) K1(x)M1(x)M1 + ...] (Sect. 2, Q1 pressure), whose entry for two
 //    corners depends only on which axes they differ in, so 8 values per element
 //    are formed in shared memory and every output node sums over its <= 8 bricks.
-//  * k_symv: batched symmetric GEMV over 32x32 upper tiles (K_II^{-1}, N_i, ...),
-//    one CTA per matrix; every warp streams its tiles global->shared with
+//  * k_symv: batched symmetric GEMV over packed upper panels (K_II^{-1}, N_i, ...),
+//    one CTA or several per matrix; every warp streams its tiles global->shared with
 //    cp.async.bulk (TMA bulk copies completing on an mbarrier), and uses each tile
 //    twice (row block and, off the diagonal, column block) with bank-conflict-free
 //    skewed shared-memory reads, so each stored element is read from HBM once.

@@ -211,6 +211,73 @@ const void* upload_dense(DeviceArena& A, const std::vector<double>& M, int prec)
   return d;
 }
 
+// The assembled rows of the subdomains, and for the dense local solver the block of K_II^{-1} of the
+// interior unknowns next to the interface. rows_entries: stored row entries per subdomain; bnd_n: unknowns of
+// that block per subdomain (dense).
+void upload_local_rows(DeviceArena& A, const HostSetup& H, int schur_prec, DevMesh& dm,
+                       std::vector<double>& rows_entries, std::vector<int>& bnd_n, cudaStream_t s) {
+  const Mesh1& M = H.mesh;
+  const bool fdm = H.local_solver == DD_LOCAL_FDM, df = schur_prec == DD_PREC_DF64;
+  const LocalRowsHost R = build_local_rows(M, H.l1, !fdm);
+  LocalRows& lr = dm.rows;
+  lr.type = A.upload(R.type, s);
+  lr.trange = A.upload(R.trange, s);
+  lr.sl_off = A.upload(R.sl_off, s);
+  lr.sl_out = A.upload(R.sl_out, s);
+  lr.sl_cnt = A.upload(R.sl_cnt, s);
+  lr.nb = A.upload(R.nb, s);
+  lr.coff = A.upload(R.coff, s);
+  if (df) {
+    std::vector<df64> cf(R.coef.size());
+#pragma omp parallel for schedule(static)
+    for (int64_t t = 0; t < (int64_t)cf.size(); ++t) cf[t] = df64_from_double(R.coef[t]);
+    lr.coef = A.upload(cf, s);
+  } else {
+    lr.coef = A.upload(R.coef, s);
+  }
+  std::vector<int64_t> boff((size_t)M.S + 1, 0);
+  rows_entries.resize(M.S);
+  for (int i = 0; i < M.S; ++i) {
+    const int nG = (int)(H.l1.goff[i + 1] - H.l1.goff[i]), nI = (int)(H.l1.ioff[i + 1] - H.l1.ioff[i]);
+    const int nB = (int)R.bnd[R.type[i]].size();
+    boff[i + 1] = boff[i] + nB;
+    lr.max_loc = std::max(lr.max_loc, nG + (fdm ? nI : nB));
+    rows_entries[i] = (double)(R.coff[i + 1] - R.coff[i]);
+  }
+  if (fdm) {
+    std::vector<int> ifree((size_t)dm.n_int);
+    const int64_t Nfx = M.fx1 - M.fx0, Nfy = M.fy1 - M.fy0;
+    for (int i = 0; i < M.S; ++i) {
+      const int16_t* code = M.lidx.data() + (size_t)i * M.NL;
+      const int I = i % M.Sx, J = (i / M.Sx) % M.Sy, K = i / (M.Sx * M.Sy);
+      for (int l = 0; l < M.NL; ++l) {
+        if (code[l] < 0) continue;
+        const int64_t x = I * M.sx + l % M.NLx - M.fx0;
+        const int64_t y = J * M.sy + (l / M.NLx) % M.NLy - M.fy0;
+        const int64_t z = K * M.sz + l / (M.NLx * M.NLy) - M.fz0;
+        ifree[H.l1.ioff[i] + code[l]] = (int)(x + Nfx * (y + Nfy * z));
+      }
+    }
+    lr.ifree = A.upload(ifree, s);
+    return;
+  }
+  lr.boff = A.upload(boff, s);
+  std::vector<std::vector<double>> blocks(M.S);
+  std::vector<const double*> mats(M.S);
+  bnd_n.resize(M.S);
+#pragma omp parallel for schedule(static)
+  for (int i = 0; i < M.S; ++i) {
+    const std::vector<int>& B = R.bnd[R.type[i]];
+    const int nb = (int)B.size(), nI = H.l1.sub[i].nI;
+    blocks[i].resize((size_t)nb * nb);
+    for (int a = 0; a < nb; ++a)
+      for (int b = 0; b < nb; ++b) blocks[i][(size_t)a * nb + b] = H.l1.sub[i].KIIinv[(size_t)B[a] * nI + B[b]];
+    mats[i] = blocks[i].data();
+    bnd_n[i] = nb;
+  }
+  dm.KBB = upload_sym(A, mats, bnd_n, df ? DD_PREC_DF64 : DD_PREC_FP64, s);
+}
+
 // the level-2 operators in the type of prec
 void upload_level2(DeviceArena& A, const HostSetup& H, int prec, DevLevel2& L, cudaStream_t s) {
   const int rp = prec == DD_PREC_FP32 ? DD_PREC_FP32 : DD_PREC_FP64;
@@ -609,8 +676,11 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
     if (A.count >= 152) {
       // FP64 products are bound by the SM's FP64 pipe (two FMAs per clock), so the launch lasts as long
       // as the SM with the most matrix parts: take the number of parts with the least work there,
-      // each further part costing the vector it stages and combines (about 4 % of a matrix).
-      // FP32 and df64 products are bound by memory: one part each.
+      // each further part costing the vector it stages and combines (about 4 % of a matrix): one part / the
+      // rule's choice for 180 matrices of 8^3 subdomains 102 / 77 us, 216 105 / 104, 320 147 / 127, 343 192 / 141,
+      // 512 232 / 214. FP32 products are bound by memory: one part. df64 products (218 unknowns) by the latency of the two
+      // CTAs that their staged blocks let on an SM; two parts paid once in four: 216 matrices 39 -> 31 us, 343
+      // 44 -> 50-58, 512 69 -> 77 (150 unknowns: 32 -> 36), so one part.
       want = 1;
       if (A.prec == DD_PREC_FP64) {
         double best = 0.0;
@@ -631,7 +701,8 @@ void tune_shapes(dd_ctx* c, cudaStream_t s) {
       zero(A.sticket, (size_t)A.count * sizeof(unsigned));
     }
   };
-  // (16^3 with 64 subdomains: one CTA per N_i left 88 SMs idle; two or more parts, 3.9 % of a solve)
+  // Fewer matrices than SMs: two or more parts each. Solves (FP32 N_i) with one part / parts: 125 subdomains of 8^3
+  // 1432 / 1233 us, 150 1721 / 1470; FP64 N_i alone, 27 subdomains 76 / 26 us, 125 79 / 63.
   split_sym(c->b1.N);
   tune_sym(c->b1.N, c->b1.goff, w.rloc, w.uloc, c->info.tune_symv_ms);
   if (c->mesh.local_solver != DD_LOCAL_FDM) {
@@ -741,7 +812,7 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
     DevMesh& dm = c->mesh;
     std::vector<double> elem_madds, elem_nbl;  // per subdomain type (for the profiling counts)
     std::vector<int> elem_type;
-    std::vector<double> rows_madds;  // per subdomain: stored row entries
+    std::vector<double> rows_madds;  // per subdomain: stored row entries (a multiply-add each)
     std::vector<int> bnd_n;          // per subdomain: interior unknowns next to the interface (dense)
     dm.nx = M.nx; dm.ny = M.ny; dm.nz = M.nz; dm.sx = M.sx; dm.sy = M.sy; dm.sz = M.sz;
     dm.Sx = M.Sx; dm.Sy = M.Sy; dm.Sz = M.Sz; dm.S = M.S;
@@ -858,68 +929,7 @@ dd_status dd_setup(const dd_mesh_desc* md, const dd_options* opt, void* stream, 
       }
       dm.KIIinv = upload_sym(A, mats, dims, opt->schur_prec == DD_PREC_DF64 ? DD_PREC_DF64 : DD_PREC_FP64, s);
     }
-    {
-            const LocalRowsHost R = build_local_rows(M, H->l1, H->local_solver != DD_LOCAL_FDM);
-            LocalRows& lr = dm.rows;
-            lr.type = A.upload(R.type, s);
-            lr.trange = A.upload(R.trange, s);
-            lr.sl_off = A.upload(R.sl_off, s);
-            lr.sl_out = A.upload(R.sl_out, s);
-            lr.sl_cnt = A.upload(R.sl_cnt, s);
-            lr.nb = A.upload(R.nb, s);
-            lr.coff = A.upload(R.coff, s);
-            if (opt->schur_prec == DD_PREC_DF64) {
-              std::vector<df64> cf(R.coef.size());
-#pragma omp parallel for schedule(static)
-              for (int64_t t = 0; t < (int64_t)cf.size(); ++t) cf[t] = df64_from_double(R.coef[t]);
-              lr.coef = A.upload(cf, s);
-            } else {
-              lr.coef = A.upload(R.coef, s);
-            }
-            if (H->local_solver == DD_LOCAL_FDM) {
-        std::vector<int> ifree((size_t)dm.n_int);
-              const int64_t Nfx = M.fx1 - M.fx0, Nfy = M.fy1 - M.fy0;
-              for (int i = 0; i < M.S; ++i) {
-                const int16_t* code = M.lidx.data() + (size_t)i * M.NL;
-                const int I = i % M.Sx, J = (i / M.Sx) % M.Sy, K = i / (M.Sx * M.Sy);
-                for (int l = 0; l < M.NL; ++l)
-                  if (code[l] >= 0) {
-                    const int a = l % M.NLx, b = (l / M.NLx) % M.NLy, q = l / (M.NLx * M.NLy);
-                    ifree[H->l1.ioff[i] + code[l]] = (int)((I * M.sx + a - M.fx0) +
-                                                           Nfx * ((J * M.sy + b - M.fy0) + Nfy * (int64_t)(K * M.sz + q - M.fz0)));
-                  }
-                  }
-              lr.ifree = A.upload(ifree, s);
-            }
-      std::vector<int64_t> boff((size_t)M.S + 1, 0);
-      for (int i = 0; i < M.S; ++i) {
-        const int nG = (int)(H->l1.goff[i + 1] - H->l1.goff[i]), nI = (int)(H->l1.ioff[i + 1] - H->l1.ioff[i]);
-        const int nB = (int)R.bnd[R.type[i]].size();
-        boff[i + 1] = boff[i] + nB;
-        lr.max_loc = std::max(lr.max_loc, nG + (H->local_solver == DD_LOCAL_FDM ? nI : nB));
-      }
-      if (H->local_solver != DD_LOCAL_FDM) {
-        lr.boff = A.upload(boff, s);
-        std::vector<std::vector<double>> blocks(M.S);
-        std::vector<const double*> mats(M.S);
-        std::vector<int> dims(M.S);
-#pragma omp parallel for schedule(static)
-        for (int i = 0; i < M.S; ++i) {
-          const std::vector<int>& B = R.bnd[R.type[i]];
-          const int nb = (int)B.size(), nI = H->l1.sub[i].nI;
-          blocks[i].resize((size_t)nb * nb);
-          for (int a = 0; a < nb; ++a)
-            for (int b = 0; b < nb; ++b) blocks[i][(size_t)a * nb + b] = H->l1.sub[i].KIIinv[(size_t)B[a] * nI + B[b]];
-          mats[i] = blocks[i].data();
-          dims[i] = nb;
-        }
-        dm.KBB = upload_sym(A, mats, dims, opt->schur_prec == DD_PREC_DF64 ? DD_PREC_DF64 : DD_PREC_FP64, s);
-        bnd_n = dims;
-      }
-      // multiply-adds and element data of the profile: the rows' entries
-            rows_madds.resize(M.S);
-            for (int i = 0; i < M.S; ++i) rows_madds[i] = (double)(R.coff[i + 1] - R.coff[i]);
-    }
+    upload_local_rows(A, *H, opt->schur_prec, dm, rows_madds, bnd_n, s);
     // ---- level-1 BDDC ----
     upload_bddc(A, H->l1, opt->precond_prec, c->b1, s);
     int pp = opt->precond_prec;
