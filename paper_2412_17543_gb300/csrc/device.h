@@ -179,15 +179,15 @@ struct DevLevel2 {
   int n3;
 };
 
-// Coarse spaces of at most this many dofs apply the level-2 BDDC as one explicit matrix
-// (built at setup). The recursive form is a chain of fourteen dependent launches of 2-8 us
+// Coarse spaces whose matrix takes at most this many bytes (4096 dofs in FP32, 2896 in FP64) apply the
+// level-2 BDDC as one explicit matrix (built at setup). The recursive form is a chain of fourteen dependent launches of 2-8 us
 // each; the matrix costs its n^2 entries from L2 or HBM. One BDDC application (4^3 subdomains), matrix / chain:
 //   one vector, FP32: 1115 dofs 39 / 92 us, 1854 40 / 94, 3249 47 / 99, 3687 51 / 99, 4615 64 / 101, 5237 88 / 101
-//   one vector, FP64: 1115 52 / 105 us, 3249 95 / 122, 3687 108 / 125, 4615 130 / 138, 5237 145 / 143
-// The line lies where FP64 still gains, before the FP64 matrix outgrows L2 (134 MB at 4096 dofs) and its
-// formation the setup (0.15 s at 3249 dofs, 0.69 s at 4615).
-constexpr int COARSE_DENSE_MAX = 4096;    // one vector: 67 MB of floats or 134 MB of doubles at most
-// Ensembles (each block of 8 rows reads all members' vectors), 32 members:
+//   one vector, FP64: 1115 59 / 105 us, 1854 70 / 116, 3249 132 / 122, 3687 136 / 125
+// FP64 loses from about 3000 dofs on. FP32 would gain up to about 5000, but the formation outgrows the rest of
+// the setup (0.15 s at 3249 dofs, 0.69 s at 4615).
+constexpr size_t COARSE_DENSE_BYTES = (size_t)64 << 20;
+// Ensembles (each block of 8 rows reads all members' vectors) up to this many dofs, 32 members:
 //   FP32: 1115 dofs 51 / 96 us, 1854 66 / 110, 3249 121 / 134, 3687 153 / 139
 //   FP64: 1115 468 / 456 us, 1854 790 / 997, 3249 1804 / 1243, 3687 2151 / 1291
 constexpr int COARSE_DENSE_MAX_B = 2048;

@@ -451,9 +451,8 @@ static bool tiles_fit(const DevLevel2& L, size_t value) {
 }
 
 bool coarse_dense_fits(const dd_ctx* c) {
-  const int n = c->b1.n_coarse;
-  if (c->levels != 3 || n == 0 || n > COARSE_DENSE_MAX) return false;
-  return tiles_fit(c->l2, c->b1.prec == DD_PREC_FP32 ? sizeof(float) : sizeof(double));
+  const size_t n = c->b1.n_coarse, value = c->b1.prec == DD_PREC_FP32 ? sizeof(float) : sizeof(double);
+  return c->levels == 3 && n > 0 && n * n * value <= COARSE_DENSE_BYTES && tiles_fit(c->l2, value);
 }
 
 // The level-2 BDDC of a small coarse space as one matrix: its columns from the operators

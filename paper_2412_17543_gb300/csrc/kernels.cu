@@ -1217,22 +1217,14 @@ void launch_dense_gemv(int n, int prec, const void* A, const double* x, double* 
   DD_CHECK_LAUNCH();
 }
 
-// Arithmetic of the explicit coarse operator: entries stored in the preconditioner's type, vectors
-// and sums in FP64 or, with FP32 entries, in df64. The products that the matrix stands for kept
-// the vectors between them in FP64; with FP32 vectors and sums here a whole FP32 application was 1.5 to 3
-// times as far from the FP64 one as through those products, in df64 it is nearer than they were.
-template <class T>
-struct CoarseOps;
-template <>
-struct CoarseOps<float> {
-  using P = PolDF;
-  __device__ static df64 entry(float a) { return {a, 0.f}; }
-};
-template <>
-struct CoarseOps<double> {
-  using P = PolF64;
-  __device__ static double entry(double a) { return a; }
-};
+// The explicit coarse operator of small coarse spaces, y = M x (row-major n x n, warp per row, sixteen
+// coalesced loads in flight per lane). The product replaces a chain of fourteen small launches on the
+// critical path beside the N_i product. Bound by the n^2 entries from HBM where that product evicts them from
+// L2, else by the latency of a row and its arithmetic.
+//
+// FP64: vectors and sums in FP64. FP32 entries: vectors and sums in df64. The products that the matrix
+// stands for kept the vectors between them in FP64; with FP32 vectors and sums here a whole FP32 application was
+// 1.5 to 3 times as far from the FP64 one as through those products, in df64 it is nearer than they were.
 
 // x_j = sum of the copies of coarse dof j
 template <class P>
@@ -1245,74 +1237,95 @@ __global__ void k_coarse_gather(int n, const int* __restrict__ ptr, const int* _
   x[j] = P::from_d(s);
 }
 
-// y = M x for the explicit coarse operator (row-major n x n, warp per row, sixteen coalesced
-// loads in flight per lane, x from L1, which holds it). The products replace a chain of fourteen small
-// launches on the critical path beside the N_i product. Bound by the n^2 entries from HBM where that product evicts
-// them from L2 (64^3, 2863 coarse dofs: 29 us beside it, 25 us with FP32 sums), else by the latency of a row
-// and the df64 arithmetic (2863 dofs on 24^3: 9.3 us; 14 us with x staged in shared memory, whose
-// copy and barrier every block paid for).
-constexpr int CG_WARPS = 4;
-constexpr int CG_BLOCKS = 8;  // per SM
 constexpr int CG_CHUNK = 16;
-template <class T>
-__global__ void __launch_bounds__(CG_WARPS * 32, CG_BLOCKS) k_coarse_gemv(
-    int n, const T* __restrict__ M, const typename CoarseOps<T>::P::V* __restrict__ x, double* __restrict__ y) {
-  using Ops = CoarseOps<T>;
-  using P = typename Ops::P;
-  using V = typename P::V;
+
+// FP64, x in shared memory. The form of k_coarse_gemv_f took 15 us instead of 40 at 1115 dofs (48^3), but
+// then Phi u_C met the N_i product in its dense part: the product 90 -> 100 us, the solve 3.74 -> 3.83 ms.
+constexpr int CG_WARPS = 8;
+__global__ void __launch_bounds__(CG_WARPS * 32) k_coarse_gemv(int n, const double* __restrict__ M,
+                                                               const double* __restrict__ x, double* __restrict__ y) {
+  extern __shared__ __align__(16) double cg_xs[];
+  for (int j = threadIdx.x; j < n; j += blockDim.x) cg_xs[j] = x[j];
+  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int i = blockIdx.x * CG_WARPS + warp; i < n; i += gridDim.x * CG_WARPS) {
-    const T* a = M + (int64_t)i * n;
-    typename P::Acc acc[4];
+    const double* a = M + (int64_t)i * n;
+    double acc[4] = {0, 0, 0, 0};
+    for (int j0 = 0; j0 < n; j0 += 32 * CG_CHUNK) {
+      double v[CG_CHUNK];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) P::init(acc[u]);
+      for (int u = 0; u < CG_CHUNK; ++u) {
+        const int j = j0 + u * 32 + lane;
+        v[u] = j < n ? a[j] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < CG_CHUNK; ++u) {
+        const int j = j0 + u * 32 + lane;
+        if (j < n) acc[u & 3] = fma(v[u], cg_xs[j], acc[u & 3]);
+      }
+    }
+    double sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) y[i] = sum;
+  }
+}
+
+// FP32 entries, x from L1 (staged in shared memory every block paid for the copy and its barrier: 2863 dofs on
+// 24^3 14 us instead of 9.3). 64^3, 2863 dofs, beside the N_i product: 29 us (25 us with FP32 sums).
+constexpr int CGF_WARPS = 4;
+constexpr int CGF_BLOCKS = 8;  // per SM
+__global__ void __launch_bounds__(CGF_WARPS * 32, CGF_BLOCKS) k_coarse_gemv_f(int n, const float* __restrict__ M,
+                                                                              const df64* __restrict__ x,
+                                                                              double* __restrict__ y) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = blockIdx.x * CGF_WARPS + warp; i < n; i += gridDim.x * CGF_WARPS) {
+    const float* a = M + (int64_t)i * n;
+    df64_acc acc[4];
     // whole chunks without bounds, and the launch bound's registers: else the compiler moves each
     // load down to its use (32 registers, 33 us instead of 29 at 64^3)
     const int n0 = n - n % (32 * CG_CHUNK);
     for (int j0 = 0; j0 < n0; j0 += 32 * CG_CHUNK) {
-      T v[CG_CHUNK];
+      float v[CG_CHUNK];
 #pragma unroll
       for (int u = 0; u < CG_CHUNK; ++u) v[u] = a[j0 + u * 32 + lane];
 #pragma unroll
-      for (int u = 0; u < CG_CHUNK; ++u) P::fma(acc[u & 3], Ops::entry(v[u]), x[j0 + u * 32 + lane]);
+      for (int u = 0; u < CG_CHUNK; ++u) acc[u & 3].fma(df64{v[u], 0.f}, x[j0 + u * 32 + lane]);
     }
     for (int j0 = n0; j0 < n; j0 += 32 * 4) {
-      T v[4];
+      float v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int j = j0 + u * 32 + lane;
-        v[u] = j < n ? a[j] : T(0);
+        v[u] = j < n ? a[j] : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int j = j0 + u * 32 + lane;
-        if (j < n) P::fma(acc[u], Ops::entry(v[u]), x[j]);
+        if (j < n) acc[u].fma(df64{v[u], 0.f}, x[j]);
       }
     }
-    const V sum = warp_sum<P>(P::add(P::add(P::get(acc[0]), P::get(acc[1])), P::add(P::get(acc[2]), P::get(acc[3]))));
-    if (lane == 0) y[i] = P::to_d(sum);
+    const df64 sum = warp_sum<PolDF>(df64_add(df64_add(acc[0].get(), acc[1].get()), df64_add(acc[2].get(), acc[3].get())));
+    if (lane == 0) y[i] = df64_to_double(sum);
   }
-}
-
-template <class T>
-static void coarse_gemv_go(int n, const T* M, const int* cptr, const int* cidx, const double* gloc, void* xs,
-                           double* y, cudaStream_t s) {
-  using P = typename CoarseOps<T>::P;
-  using V = typename P::V;
-  k_coarse_gather<P><<<(n + 127) / 128, 128, 0, s>>>(n, cptr, cidx, gloc, static_cast<V*>(xs));
-  DD_CHECK_LAUNCH();
-  const int blocks = std::min(152 * CG_BLOCKS, (n + CG_WARPS - 1) / CG_WARPS);
-  k_coarse_gemv<T><<<blocks, CG_WARPS * 32, 0, s>>>(n, M, static_cast<const V*>(xs), y);
-  DD_CHECK_LAUNCH();
 }
 
 void launch_coarse_gemv(int n, int prec, const void* M, const int* cptr, const int* cidx, const double* gloc,
                         void* xs, double* y, cudaStream_t s) {
   if (n == 0) return;
-  if (prec == DD_PREC_FP32)
-    coarse_gemv_go<float>(n, (const float*)M, cptr, cidx, gloc, xs, y, s);
-  else
-    coarse_gemv_go<double>(n, (const double*)M, cptr, cidx, gloc, xs, y, s);
+  if (prec == DD_PREC_FP32) {
+    k_coarse_gather<PolDF><<<(n + 127) / 128, 128, 0, s>>>(n, cptr, cidx, gloc, static_cast<df64*>(xs));
+    DD_CHECK_LAUNCH();
+    const int blocks = std::min(152 * CGF_BLOCKS, (n + CGF_WARPS - 1) / CGF_WARPS);
+    k_coarse_gemv_f<<<blocks, CGF_WARPS * 32, 0, s>>>(n, static_cast<const float*>(M), static_cast<const df64*>(xs), y);
+  } else {
+    k_coarse_gather<PolF64><<<(n + 127) / 128, 128, 0, s>>>(n, cptr, cidx, gloc, static_cast<double*>(xs));
+    DD_CHECK_LAUNCH();
+    const int blocks = std::min(152 * 4, (n + CG_WARPS - 1) / CG_WARPS);
+    k_coarse_gemv<<<blocks, CG_WARPS * 32, (size_t)n * sizeof(double), s>>>(n, static_cast<const double*>(M),
+                                                                           static_cast<const double*>(xs), y);
+  }
+  DD_CHECK_LAUNCH();
 }
 
 __global__ void k_map_gather(int64_t n, const int* __restrict__ map, const double* __restrict__ in,
