@@ -518,8 +518,9 @@ static void symm_go(const SymTiles& A, const int64_t* voff, const void* in, void
   max_smem(k_symm_b<T, W>, smem);
   k_symm_b<T, W><<<A.count, W * 32, smem, s>>>(A, voff, (const T*)in, (T*)out);
 }
-// Warps per matrix: as many as block rows, 4, 8 or 16. A warp without a block row takes room from other
-// matrices (FP64, 512 matrices: SYMMFIG
+// Warps per matrix: 4, 8 or 16 by block rows, since a warp without a block row takes room from other matrices.
+// FP64, 4 / 8 / 16 warps: 512 matrices of 4 block rows 599 / - / 1040 us, 512 of 5 1148 / 1039 / 1470, 216 of 7
+// 1191 / 861 / 984, 512 of 13 5825 / - / 4914. With fewer matrices than SMs (level 2) room is no matter: sixteen.
 template <class T>
 static void symm_warps(const SymTiles& A, const int64_t* voff, const void* in, void* out, int npad, cudaStream_t s) {
   const size_t smem = (size_t)npad * BW * sizeof(T);

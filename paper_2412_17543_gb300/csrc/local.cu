@@ -348,8 +348,9 @@ constexpr int LBS = 128;  // threads of the single-vector kernel: 98 line halves
                           // slices of a pass at once) took 47 us instead of 26 on 512 subdomains
 
 // One vector. 12.9 KB of shared memory per 8^3 subdomain (a compact vector and one interior buffer 8.6 KB, the
-// staged bases 4.3 KB): 16 CTAs of 128 threads fill an SM's 2048 threads and 206 of its 228 KB, and their phases
-// overlap; the rows' coefficients stream from HBM (about 77 KB per 8^3 subdomain).
+// staged bases 4.3 KB) and 72 registers a thread (95 in the df64 recovery): registers let seven (five) CTAs on an SM,
+// whose phases overlap; the rows' coefficients stream from HBM (about 77 KB per 8^3 subdomain). Bound by
+// latency, of instruction fetches first of all (the unrolled products), then of the coefficients.
 template <class P, int MODE>
 __global__ void __launch_bounds__(LBS) k_local_apply(DevMesh m, const double* __restrict__ xg,
                                                      const double* __restrict__ f, double* __restrict__ out) {

@@ -1,5 +1,5 @@
-"""dd_schur_apply_noalloc with the dense local solver (coefficient varying inside the subdomains): fewer
-subdomains than SMs and more, where the context's own product with K_II^{-1} is divided among several
+"""dd_schur_apply_noalloc with the dense local solver (coefficient varying inside the subdomains): more
+subdomains than SMs, and fewer, where the context's own product with K_II^{-1} is divided among several
 CTAs per matrix. The entry point promises no shared state but its scratch array, so it also runs beside
 dd_schur_apply of the same context on another stream. Tolerances of test_gpu_parity.py: FP64 1e-12 of
 the largest entry, df64 1e-11.
