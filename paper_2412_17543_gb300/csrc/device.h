@@ -188,8 +188,9 @@ struct DevLevel2 {
 // the setup (0.15 s at 3249 dofs, 0.69 s at 4615).
 constexpr size_t COARSE_DENSE_BYTES = (size_t)64 << 20;
 // Ensembles (each block of 8 rows reads all members' vectors) up to this many dofs, 32 members:
-//   FP32: 1115 dofs 51 / 96 us, 1854 66 / 110, 3249 121 / 134, 3687 153 / 139
-//   FP64: 1115 468 / 456 us, 1854 790 / 997, 3249 1804 / 1243, 3687 2151 / 1291
+//   FP32: 1115 dofs 51 / 101 us, 1854 70 / 119, 2143 75 / 121, 2863 103 / 141, 3249 114 / 149, 3687 141 / 145
+//   FP64: 1115 383 / 427 us, 1854 632 / 1042, 2143 747 / 1087, 2863 1070 / 1208
+// (drawn when FP64 still lost from about 2500 dofs on; it could lie at the bytes above now)
 constexpr int COARSE_DENSE_MAX_B = 2048;
 
 // Scratch buffers of the operators (device).
